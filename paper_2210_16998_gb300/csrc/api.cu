@@ -391,7 +391,6 @@ struct tpg_cfg {
     unsigned long long spin_ns = SPIN_LIMIT_NS;  // limit of each grid-barrier wait of the frontier launch
     // generic scratch
     DevBuf s_keys[2], s_refs[2], s_len, s_tmp, s_i32[3], s_i64[4];
-    DevBuf rank_cnt, rank_pre[2], rank_noff, rank_bsum;  // PP ranking scratch
     DevBuf pp_ends;  // (first, last) local vertex of each cached PP, for the TP lengths
     DevBuf tp_key_off, tp_key;  // packed comparison keys of the TPs being sorted
 
@@ -411,9 +410,9 @@ struct tpg_cfg {
         cudaGraphExec_t exec = nullptr;
         cudaStream_t own_stream = nullptr;
         DevBuf seg, ppseg, tfl[2], tvis[2], tcnt[2];
-        DevBuf lvl_pp_off, keys[2], refs[2], len, scan_tmp, pp_graph, tp_len, run_start, run_rank, tp_graph0,
+        DevBuf lvl_pp_off, refs[2], len, scan_tmp, pp_graph, tp_len, run_start, run_rank, tp_graph0,
             run_base, nruns, bounds0, tp_off0, tp_vert0, perm[2], keep, keep_off, keep_rank, tp_graph, counts,
-            key_off, key, rank_cnt, rank_pre[2], rank_noff, rank_bsum;
+            key_off, key;
         Block *pp_off = nullptr, *pp_vert = nullptr, *pp_gptr = nullptr;
         Block *tp_off = nullptr, *tp_vert = nullptr, *tp_gptr = nullptr;
         long long seg_cap = 0, pp_cap = 0, lvl_cap = 0;
@@ -486,11 +485,10 @@ void release_plan(tpg_cfg *g) {
     if (p.exec) cudaGraphExecDestroy(p.exec);
     p.exec = nullptr;
     DevBuf *all[] = {&p.seg, &p.ppseg, &p.tfl[0], &p.tfl[1], &p.tvis[0], &p.tvis[1], &p.tcnt[0], &p.tcnt[1], &p.lvl_pp_off,
-                     &p.keys[0], &p.keys[1], &p.refs[0], &p.refs[1], &p.len, &p.scan_tmp, &p.pp_graph, &p.tp_len,
+                     &p.refs[0], &p.refs[1], &p.len, &p.scan_tmp, &p.pp_graph, &p.tp_len,
                      &p.run_start, &p.run_rank, &p.tp_graph0, &p.run_base, &p.nruns, &p.bounds0, &p.tp_off0,
                      &p.tp_vert0, &p.perm[0], &p.perm[1], &p.keep, &p.keep_off, &p.keep_rank, &p.tp_graph,
-                     &p.counts, &p.key_off, &p.key, &p.rank_cnt, &p.rank_pre[0], &p.rank_pre[1],
-                     &p.rank_noff, &p.rank_bsum};
+                     &p.counts, &p.key_off, &p.key};
     for (DevBuf *b : all) release(g, *b);
     Block *bl[] = {p.pp_off, p.pp_vert, p.pp_gptr, p.tp_off, p.tp_vert, p.tp_gptr};
     for (Block *b : bl) block_unref(b);
@@ -512,8 +510,7 @@ void destroy_cfg(tpg_cfg *g) {
                      &g->pre_seq, &g->suf_seq, &g->tfl[0], &g->tfl[1], &g->tvis[0], &g->tvis[1], &g->tcnt[0], &g->tcnt[1],
                      &g->levels, &g->agg, &g->ctl, &g->s_keys[0], &g->s_keys[1],
                      &g->s_refs[0], &g->s_refs[1], &g->s_len, &g->s_tmp, &g->s_i32[0], &g->s_i32[1],
-                     &g->s_i32[2], &g->s_i64[0], &g->s_i64[1], &g->s_i64[2], &g->s_i64[3], &g->rank_cnt,
-                     &g->rank_pre[0], &g->rank_pre[1], &g->rank_noff, &g->rank_bsum, &g->pp_ends, &g->tp_key_off, &g->tp_key,
+                     &g->s_i32[2], &g->s_i64[0], &g->s_i64[1], &g->s_i64[2], &g->s_i64[3], &g->pp_ends, &g->tp_key_off, &g->tp_key,
                      &g->trace};
     for (DevBuf *b : all) release(g, *b);
     for (auto &b : g->node_segs) release(g, b);
@@ -679,6 +676,10 @@ int alloc_fixed_workspace(tpg_cfg *g) {
     return TPG_OK;
 }
 
+// A node segment holds its nodes and then their places.
+constexpr size_t NODE_BYTES = 2 * sizeof(int2);
+long long seg_nodes(const DevBuf &b) { return (long long)(b.bytes / NODE_BYTES); }
+
 // Ping-pong frontier buffers of capacity g->lvl_cap.
 int alloc_frontier(tpg_cfg *g) {
     for (int b = 0; b < 2; ++b) {
@@ -719,7 +720,7 @@ int prepare_segments(tpg_cfg *g, std::vector<DevBuf> &segs, size_t elem, long lo
 // more, which leaves the rest of the call (ordering and materialisation,
 // sized by the exact counts) as much room again.
 int alloc_enumeration_once(tpg_cfg *g) {
-    int rc = prepare_segments(g, g->node_segs, sizeof(int2), g->node_cap);
+    int rc = prepare_segments(g, g->node_segs, NODE_BYTES, g->node_cap);
     if (rc == TPG_OK) rc = prepare_segments(g, g->pp_segs, sizeof(int), g->pp_cap);
     if (rc == TPG_OK) rc = alloc_frontier(g);
     return rc;
@@ -790,7 +791,8 @@ int enumerate_levels(tpg_cfg *g) {
         EnumArgs a{};
         a.g = g->gd;
         a.seg = seg.as<int2>();
-        a.seg_cap = (long long)(seg.bytes / sizeof(int2));
+        a.seg_cap = seg_nodes(seg);
+        a.seg_place = a.seg + a.seg_cap;
         a.next_nodes = next_override;
         a.pp_seg = ppseg.as<int>();
         a.pp_seg_cap = (long long)(ppseg.bytes / sizeof(int));
@@ -858,8 +860,8 @@ int enumerate_levels(tpg_cfg *g) {
         next_override = nullptr;
         if (err & ERR_OVF_NODES) {
             long long total = 0;
-            for (auto &b : g->node_segs) total += (long long)(b.bytes / sizeof(int2));
-            RC(push_segment(g, g->node_segs, sizeof(int2), std::max(L.children, 3 * total)));
+            for (auto &b : g->node_segs) total += seg_nodes(b);
+            RC(push_segment(g, g->node_segs, NODE_BYTES, std::max(L.children, 3 * total)));
             next_override = g->node_segs.back().as<int2>();
         }
         if (err & ERR_OVF_PP) {
@@ -928,7 +930,7 @@ int run_prime_paths(tpg_cfg *g) {
     g->stats.prime_paths = P;
     g->stats.pp_vertices = V;
     g->stats.bitset_words = g->W;
-    g->stats.arena_bytes_used = nodes * (long long)sizeof(int2);
+    g->stats.arena_bytes_used = nodes * (long long)NODE_BYTES;
     long long seg_bytes = 0;
     for (auto &b : g->node_segs) seg_bytes += (long long)b.bytes;
     g->stats.arena_bytes_alloc = seg_bytes;
@@ -962,36 +964,16 @@ int run_prime_paths(tpg_cfg *g) {
         CK(pp_materialize(nullptr, refs, k, P, (const long long *)off->p, dlev, g->max_levels, g->gd, (int *)vert->p,
                           pgraph ? (int *)pgraph->p : nullptr, s, ends));
     } else {
-        // canonical order by pre-order rank in the arena's prefix tree
+        // canonical order from the places in the arena's prefix tree
         RC(ensure(g, g->s_refs[0], sizeof(long long) * P));
-        RC(ensure(g, g->s_len, sizeof(long long) * (P + 1)));
-        RC(ensure(g, g->s_tmp, sizeof(long long) * scan_tmp_elems(P + 1)));
-        RC(ensure(g, g->rank_cnt, sizeof(int) * nodes));
-        for (int b = 0; b < 2; ++b) RC(ensure(g, g->rank_pre[b], sizeof(int) * peak));
-        RC(ensure(g, g->rank_noff, sizeof(long long) * (g->max_levels + 8)));
-        RC(ensure(g, g->rank_bsum, sizeof(long long) * rank_pps_grid(g->num_sms)));
-        CK(cudaMemsetAsync(g->ctl.p, 0, CTL_BYTES, s));
-        CK(cudaMemsetAsync(g->rank_cnt.p, 0, sizeof(int) * nodes, s));
-        RankArgs r{};
-        r.cnt_zeroed = 1;
+        PlaceArgs r{};
         r.levels = dlev;
         r.max_levels = g->max_levels;
-        r.cnt = g->rank_cnt.as<int>();
-        r.cnt_cap = nodes;
-        r.pre[0] = g->rank_pre[0].as<int>();
-        r.pre[1] = g->rank_pre[1].as<int>();
-        r.pre_cap = peak;
-        r.noff = g->rank_noff.as<long long>();
-        r.bsum = g->rank_bsum.as<long long>();
         r.refs = g->s_refs[0].as<long long>();
-        r.refs_cap = P;
-        r.bar = (unsigned *)(g->ctl.as<char>() + CTL_RANK_BAR_OFFSET);
-        r.err = g->ctl.as<int>();
-        CK(rank_pps(r, g->num_sms, s));
-        const int cur = 0;
-        const long long *refs = g->s_refs[cur].as<long long>();
-        CK(pp_lengths(refs, P, g->s_len.as<long long>(), s));
-        CK(scan_i64(g->s_len.as<long long>(), (long long *)off->p, P, g->s_tmp.as<long long>(), s));
+        r.off = (long long *)off->p;
+        r.cap = P;
+        CK(place_pps(r, g->num_sms, s));
+        const long long *refs = g->s_refs[0].as<long long>();
         CK(pp_materialize(refs, nullptr, 0, P, (const long long *)off->p, dlev, g->max_levels, g->gd, (int *)vert->p,
                           pgraph ? (int *)pgraph->p : nullptr, s, ends));
     }
@@ -1004,11 +986,8 @@ int run_prime_paths(tpg_cfg *g) {
         CK(cudaMemcpyAsync(gptr->p, h, 2 * sizeof(long long), cudaMemcpyHostToDevice, s));
     }
     CK(cudaEventRecord(g->ev[3], s));
-    CK(cudaMemcpyAsync(g->h_small, g->ctl.p, sizeof(int), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
     cudaEventElapsedTime(&g->stats.t_order_ms, g->ev[2], g->ev[3]);
-    if (g->h_small[0] & ERR_TIMEOUT) return TPG_ETIMEOUT;
-    if (g->h_small[0]) return TPG_ECUDA;  // the ranking found its scratch too small
     g->P = P;
     g->V = V;
     g->pp_valid = true;
@@ -1339,13 +1318,12 @@ int capture_plan(tpg_cfg *g) {
     p.pp_cap = std::max(p.pp_cap, p.P_cap);
     const long long Pc = p.P_cap;
     const int W = g->W;
-    RC(ensure(g, p.seg, sizeof(int2) * p.seg_cap));
+    RC(ensure(g, p.seg, NODE_BYTES * p.seg_cap));
     RC(ensure(g, p.ppseg, sizeof(int) * p.pp_cap));
     for (int b = 0; b < 2; ++b) {
         RC(ensure(g, p.tfl[b], sizeof(int2) * p.lvl_cap));
         RC(ensure(g, p.tvis[b], sizeof(unsigned) * (size_t)W * p.lvl_cap));
         RC(ensure(g, p.tcnt[b], sizeof(unsigned short) * p.lvl_cap));
-        RC(ensure(g, p.keys[b], sizeof(int) * Pc));
         RC(ensure(g, p.refs[b], sizeof(long long) * Pc));
         RC(ensure(g, p.perm[b], sizeof(long long) * Pc));
     }
@@ -1371,10 +1349,6 @@ int capture_plan(tpg_cfg *g) {
     const long long K_cap = p.TV0_cap / (64 / key_bits) + Pc + 1;
     RC(ensure(g, p.key_off, sizeof(long long) * (Pc + 1)));
     RC(ensure(g, p.key, sizeof(unsigned long long) * K_cap));
-    RC(ensure(g, p.rank_cnt, sizeof(int) * p.seg_cap));
-    for (int b = 0; b < 2; ++b) RC(ensure(g, p.rank_pre[b], sizeof(int) * p.lvl_cap));
-    RC(ensure(g, p.rank_noff, sizeof(long long) * (g->max_levels + 8)));
-    RC(ensure(g, p.rank_bsum, sizeof(long long) * rank_pps_grid(g->num_sms)));
     RC(alloc_fixed_workspace(g));
     p.pp_off = block_new(g->fns, sizeof(long long) * (Pc + 1), s);
     p.pp_vert = block_new(g->fns, sizeof(int) * p.V_cap, s);
@@ -1389,6 +1363,7 @@ int capture_plan(tpg_cfg *g) {
     a.g = g->gd;
     a.seg = p.seg.as<int2>();
     a.seg_cap = p.seg_cap;
+    a.seg_place = a.seg + a.seg_cap;
     a.next_nodes = nullptr;
     a.pp_seg = p.ppseg.as<int>();
     a.pp_seg_cap = p.pp_cap;
@@ -1421,11 +1396,9 @@ int capture_plan(tpg_cfg *g) {
     m.TV0_cap = p.TV0_cap;
     m.TV_cap = p.TV_cap;
     m.num_sms = g->num_sms;
-    m.bar = (unsigned *)(g->ctl.as<char>() + 128);
     m.tp_rounds = gm_tp_rounds(g->maxn);
     m.lvl_pp_off = p.lvl_pp_off.as<long long>();
     for (int b = 0; b < 2; ++b) {
-        m.keys[b] = p.keys[b].as<int>();
         m.refs[b] = p.refs[b].as<long long>();
         m.perm[b] = p.perm[b].as<long long>();
     }
@@ -1456,14 +1429,6 @@ int capture_plan(tpg_cfg *g) {
     m.tp_graph = p.tp_graph.as<int>();
     m.tp_gptr = (long long *)p.tp_gptr->p;
     m.counts = p.counts.as<GmCounts>();
-    m.rank_cnt = p.rank_cnt.as<int>();
-    m.rank_cnt_cap = p.seg_cap;
-    m.rank_pre[0] = p.rank_pre[0].as<int>();
-    m.rank_pre[1] = p.rank_pre[1].as<int>();
-    m.rank_pre_cap = p.lvl_cap;
-    m.rank_noff = p.rank_noff.as<long long>();
-    m.rank_bsum = p.rank_bsum.as<long long>();
-    m.rank_bar = (unsigned *)(g->ctl.as<char>() + CTL_RANK_BAR_OFFSET);
     CK(cudaStreamSynchronize(s));
 
     cudaGraph_t graph = nullptr;
@@ -2797,8 +2762,7 @@ int tpg_sizer_presize(tpg_sizer *z, tpg_cfg *g, double margin, int64_t *caps_out
     const double lvl = nodes * std::min(1.0, rp * margin), TV0 = V * (z->r_tv0 > 0 ? z->r_tv0 : 2.0) * margin,
                  TV = V * (z->r_tv > 0 ? z->r_tv : 2.0) * margin;
     // a capture holds all of these at once: keep its buffers (per path: arena
-    // node and rank count, 12 bytes; per frontier slot: both ping-pong halves
-    // and rank prefixes; per PP: its reference and ~170 bytes of ordering, TP
+    // node and place, 16 bytes; per frontier slot: both ping-pong halves; per PP: its reference and ~170 bytes of ordering, TP
     // and output workspace; PP and TP vertices and TP merge keys; 25% growth
     // slack of every buffer) within half of the free device memory; smaller
     // capacities only cost a fallback to the exact path
@@ -2808,7 +2772,7 @@ int tpg_sizer_presize(tpg_sizer *z, tpg_cfg *g, double margin, int64_t *caps_out
         free_b = 0;
     }
     const double bytes =
-        1.25 * (12.0 * nodes + (2.0 * (sizeof(int2) + 4.0 * g->W + sizeof(unsigned short)) + 8.0) * lvl +
+        1.25 * ((double)NODE_BYTES * nodes + 2.0 * (sizeof(int2) + 4.0 * g->W + sizeof(unsigned short)) * lvl +
                 (sizeof(int) + 170.0) * P + 4.0 * V + 6.0 * TV0 + 4.0 * TV);
     const double f = free_b ? std::min(1.0, 0.5 * (double)free_b / bytes) : 1.0;
     // list sizes also stay below 2^31 (a larger need falls back as well)

@@ -36,7 +36,8 @@ struct LevelRec {
     int *pp;                // the level's first PP reference
     long long pp_count;     // PPs found in the level
     long long children;     // nodes of the next level (exact, also on overflow)
-    long long pad[3];
+    int2 *place;            // per node: where its children start in the next level, PPs before it in its level
+    long long pad[2];
 };
 
 // Device view of one handle's graph(s): the union of all graphs with global

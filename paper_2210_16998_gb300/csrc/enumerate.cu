@@ -68,6 +68,7 @@ __global__ void init_level1_kernel(EnumArgs a) {
         r.nodes = a.seg;
         r.count = g.N;
         r.pp = a.pp_seg;
+        r.place = a.seg_place;
         a.levels[1] = r;
     }
 }
@@ -191,6 +192,7 @@ __device__ __forceinline__ int enum_prologue(const EnumArgs &a) {
     long long count = __ldcg(&a.levels[1].count);
     int2 *lnodes = (int2 *)__ldcg((const unsigned long long *)&a.levels[1].nodes);
     int *lpp = (int *)__ldcg((const unsigned long long *)&a.levels[1].pp);
+    int2 *lplace = a.seg_place;
     while (count > 0 && count <= (long long)BLOCK * PI && k + 1 < a.max_levels) {
         const unsigned long long t_start = a.trace ? global_ns() : 0ull;
         int2 *const next = lnodes + count;
@@ -249,6 +251,7 @@ __device__ __forceinline__ int enum_prologue(const EnumArgs &a) {
                 r.nodes = next;
                 r.count = C;
                 r.pp = lpp + P;
+                r.place = a.seg_place ? lplace + count : nullptr;
                 a.levels[k + 1] = r;
             }
         }
@@ -258,6 +261,7 @@ __device__ __forceinline__ int enum_prologue(const EnumArgs &a) {
         for (int j = 0; j < PI; ++j) {
             const int i = lo + j;
             if (i >= hi) continue;
+            if (lplace) lplace[i] = make_int2(pos_c, pos_p);
             if (cw[j] & CNT_PP) lpp[pos_p++] = i;
             if (cnt_children(cw[j]) == 0) continue;
             auto child = [&](int w) {
@@ -294,6 +298,7 @@ __device__ __forceinline__ int enum_prologue(const EnumArgs &a) {
             atomicAdd(tr + 3, 1ull);
         }
         __syncthreads();  // this level's records are read by other threads of the block next
+        if (lplace) lplace += count;
         count = C;
         lnodes = next;
         lpp += P;
@@ -490,6 +495,7 @@ __global__ void __launch_bounds__(BLOCK, W <= 8 ? 1024 / BLOCK : 1) enumerate_ke
     long long count = __ldcg(&a.levels[k_first].count);
     int2 *lnodes = (int2 *)__ldcg((const unsigned long long *)&a.levels[k_first].nodes);
     int *lpp = (int *)__ldcg((const unsigned long long *)&a.levels[k_first].pp);
+    int2 *lplace = (int2 *)__ldcg((const unsigned long long *)&a.levels[k_first].place);
     for (int k = k_first; k + 1 < a.max_levels && count > 0; ++k) {
         int2 *const next = (k == a.start_level && a.next_nodes) ? a.next_nodes : lnodes + count;
         const long long next_off = next - a.seg;  // offset of the next level in the segment
@@ -549,6 +555,7 @@ __global__ void __launch_bounds__(BLOCK, W <= 8 ? 1024 / BLOCK : 1) enumerate_ke
                 r.nodes = next;
                 r.count = C;
                 r.pp = lpp + P;
+                r.place = a.seg_place ? a.seg_place + next_off : nullptr;
                 a.levels[k + 1] = r;
             }
         }
@@ -714,6 +721,7 @@ __global__ void __launch_bounds__(BLOCK, W <= 8 ? 1024 / BLOCK : 1) enumerate_ke
                         }
                     }
                     const int excl = x - nch;
+                    if (lplace && i < hi) lplace[i] = make_int2(pos_c + excl, pos_p + __popc(ppm & lt_mask));
                     int vb_l = 0, e0_l = 0;
                     if (nch > 0) {
                         vb_l = g.vgraph ? __ldg(g.vbase + __ldg(g.vgraph + first[j])) : 0;
@@ -954,6 +962,7 @@ __global__ void __launch_bounds__(BLOCK, W <= 8 ? 1024 / BLOCK : 1) enumerate_ke
         count = C;
         lnodes = next;
         lpp += P;
+        if (lplace) lplace = a.seg_place + next_off;
     }
 }
 

@@ -3,13 +3,7 @@
 // graph or a batch of thousands) is a fixed sequence of launches that can be
 // captured once into a CUDA graph and replayed.
 //
-// Prime-path order (kernel (e) for PPs): the PPs of each frontier level form
-// a sorted run (levels are lexicographically ordered and PPs form an
-// antichain of the prefix tree).  One cooperative persistent kernel walks
-// the levels from the deepest up: the run accumulated so far is keyed by
-// each element's ancestor index at the current level and merged with that
-// level's PPs (whose keys are their own indices; the two never tie), with a
-// bounded grid barrier between the steps.
+// Prime-path order (kernel (e) for PPs): place_pps, as in the host-driven path.
 //
 // Test-path order: the TPs of one graph that share a first vertex form a
 // sorted run; runs are merged pairwise inside each graph in
@@ -153,13 +147,6 @@ __device__ __forceinline__ long long gm_P(const GmArgs &a) {
     const GmCounts *c = a.counts;
     if (c->flags & (GM_ENUM_FAILED | GM_OVF_PP | GM_OVF_PPV)) return 0;
     return clampc(c->P, a.P_cap);
-}
-
-__global__ void __launch_bounds__(GMB) gm_pp_lengths(GmArgs a) {
-    const long long P = gm_P(a);
-    const long long *refs = a.refs[a.counts->pp_buf];
-    for (long long i = blockIdx.x * (long long)GMB + threadIdx.x; i < P; i += (long long)gridDim.x * GMB)
-        a.len[i] = refs[i] >> 32;
 }
 
 constexpr int GM_MAT_WARPS = 8;
@@ -424,27 +411,15 @@ cudaError_t gm_enqueue_pp(const GmArgs &a, cudaStream_t s) {
     const unsigned grid = stream_grid(a.num_sms);
     gm_level_summary<<<1, GMB, 0, s>>>(a);
     note_launch();
-    RankArgs r{};
+    PlaceArgs r{};
     r.levels = a.levels;
     r.max_levels = a.max_levels;
-    r.cnt = a.rank_cnt;
-    r.cnt_cap = a.rank_cnt_cap;
-    r.pre[0] = a.rank_pre[0];
-    r.pre[1] = a.rank_pre[1];
-    r.pre_cap = a.rank_pre_cap;
-    r.noff = a.rank_noff;
-    r.bsum = a.rank_bsum;
     r.refs = a.refs[0];  // counts->pp_buf stays 0
-    r.refs_cap = a.P_cap;
-    r.bar = a.rank_bar;
-    r.err = &a.counts->flags;  // any flag sends the replay to the exact path
+    r.off = a.pp_off;
+    r.cap = a.P_cap;
     r.skip = &a.counts->flags;
     r.skip_mask = GM_ENUM_FAILED | GM_OVF_PP | GM_OVF_PPV;
-    cudaError_t e = rank_pps(r, a.num_sms, s);
-    if (e != cudaSuccess) return e;
-    gm_pp_lengths<<<grid, GMB, 0, s>>>(a);
-    note_launch();
-    e = gm_scan<long long>(a.len, a.pp_off, &a.counts->P, a.P_cap, a.scan_tmp, nullptr, a.num_sms, s);
+    cudaError_t e = place_pps(r, a.num_sms, s);
     if (e != cudaSuccess) return e;
     if (a.g.maxn <= MAT_SMALL_N) gm_materialize<2, unsigned char><<<grid, GM_MAT_WARPS * 32, 0, s>>>(a);
     else gm_materialize<1, unsigned short><<<grid, GM_MAT_WARPS * 32, 0, s>>>(a);

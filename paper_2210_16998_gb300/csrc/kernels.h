@@ -42,17 +42,16 @@ __host__ __device__ inline int cnt_children(unsigned cw) {
 #endif
 }
 // control block of a launch (err, stop_level, ...); the frontier's grid
-// barrier lives at CTL_BAR_OFFSET, the PP ranking's at CTL_RANK_BAR_OFFSET,
-// other cooperative kernels use offset 128
+// barrier lives at CTL_BAR_OFFSET
 constexpr int CTL_BYTES = 1024;
 constexpr int CTL_BAR_OFFSET = 256;
-constexpr int CTL_RANK_BAR_OFFSET = 512;  // grid barrier of the PP ranking
 constexpr int CTL_HANDOFF_OFFSET = 64;    // level a frontier launch's single-block start hands to the grid
 
 struct EnumArgs {
     GraphDev g;
     int2 *seg;               // current arena segment (nodes {last, parent})
     long long seg_cap;
+    int2 *seg_place;         // the segment's places, node i's at [i] (null: not kept; see place_pps)
     int2 *next_nodes;        // where level start_level+1 starts (null: right after level start_level)
     int *pp_seg;             // current PP-reference segment
     long long pp_seg_cap;
@@ -129,28 +128,19 @@ cudaError_t pp_materialize(const long long *refs, const int *single_refs, int si
                            int *out_vertices, int *out_graph, cudaStream_t s, int2 *out_ends = nullptr);
 cudaError_t graph_ptr_from_ids(const int *ids, long long n, int G, long long *ptr, cudaStream_t s);
 
-// canonical PP order by pre-order rank in the arena's prefix tree (one
-// cooperative launch; all level sizes are read from the device level table)
-struct RankArgs {
+// canonical PP order: every PP's place from the arena's nodes and places (one
+// launch without waiting between blocks; all level sizes are read from the
+// device level table)
+struct PlaceArgs {
     const LevelRec *levels;
     int max_levels;
-    int *cnt;             // [cnt_cap] >= all simple paths: per-node PP counts
-    long long cnt_cap;
-    int *pre[2];          // [pre_cap] each >= the largest level: ranks of two consecutive levels
-    long long pre_cap;
-    long long *noff;      // [max_levels + 8]: node offset of each level, then totals
-    long long *bsum;      // [grid]
-    long long *refs;      // [refs_cap]: the sorted PP references (level << 32 | index)
-    long long refs_cap;
-    unsigned *bar;        // grid barrier: bar[0] is its arrival counter (zeroed)
-    int *err;             // ERR_INVAL (a capacity too small), ERR_TIMEOUT
+    long long *refs;      // [cap]: the sorted PP references (level << 32 | index)
+    long long *off;       // [cap + 1]: first vertex of every PP, then the total
+    long long cap;
     const int *skip;      // optional: nothing is done when (*skip & skip_mask)
     int skip_mask;
-    int cnt_zeroed;       // 1: cnt[0 .. all simple paths) is zero at launch (else the launch zeroes it)
 };
-// scratch of rank_pps beyond cnt/pre: noff [max_levels + 8], bsum [rank_pps_grid(num_sms)]
-int rank_pps_grid(int num_sms);
-cudaError_t rank_pps(const RankArgs &a, int num_sms, cudaStream_t s);
+cudaError_t place_pps(const PlaceArgs &a, int num_sms, cudaStream_t s);
 
 // graphmode.cu: the device-driven pipeline captured into a CUDA graph
 enum : int {
@@ -175,9 +165,7 @@ struct GmArgs {
     const int *enum_err;
     long long P_cap, V_cap, TV0_cap, TV_cap;
     int num_sms, tp_rounds;
-    unsigned *bar;          // grid barrier of the ordering kernel (zeroed)
     long long *lvl_pp_off;  // [max_levels+1]
-    int *keys[2];
     long long *refs[2];
     long long *len;         // [P_cap]
     long long *scan_tmp;    // gm_scan_tmp_elems(P_cap)
@@ -205,13 +193,6 @@ struct GmArgs {
     int *tp_graph;          // [P_cap]
     long long *tp_gptr;     // [G+1]
     GmCounts *counts;
-    // PP ranking scratch (rank_pps)
-    int *rank_cnt;
-    long long rank_cnt_cap;
-    int *rank_pre[2];
-    long long rank_pre_cap;
-    long long *rank_noff, *rank_bsum;
-    unsigned *rank_bar;
 };
 int gm_tp_rounds(int maxn);
 size_t gm_scan_tmp_elems(long long n_cap);
