@@ -260,6 +260,7 @@ struct HandlePool {
     std::mutex mu;
     std::vector<void *> small;
     std::map<int, std::vector<cudaEvent_t>> events;
+    std::map<int, std::vector<cudaStream_t>> sides;
 
     void *get_small() {
         std::lock_guard<std::mutex> lk(mu);
@@ -279,6 +280,25 @@ struct HandlePool {
         if (!p) return;
         std::lock_guard<std::mutex> lk(mu);
         small.push_back(p);
+    }
+    // a stream of device `dev` for work beside the caller's stream within one
+    // call (null if none can be made); as many exist as calls ever ran at once
+    cudaStream_t get_side(int dev) {
+        std::lock_guard<std::mutex> lk(mu);
+        auto &v = sides[dev];
+        cudaStream_t s = nullptr;
+        if (!v.empty()) {
+            s = v.back();
+            v.pop_back();
+        } else if (cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        return s;
+    }
+    void put_side(int dev, cudaStream_t s) {
+        std::lock_guard<std::mutex> lk(mu);
+        sides[dev].push_back(s);
     }
     // n events of the current device `dev`; false (and none taken) on failure
     bool get_events(int dev, cudaEvent_t *ev, int n) {
@@ -375,11 +395,13 @@ struct tpg_cfg {
 
     int N = 0, G = 0, maxn = 0, W = 1, max_levels = 0;
     long long M = 0, max_arcs = 0;  // arcs in total and in the graph with the most
+    long long tbl = 0;              // entries of the BFS tables
     std::vector<int> h_vbase;
 
     DevBuf rp, col, prp, pcol, vgraph, vbase, entry, exitv, tbl_base, dist, pred;
     DevBuf pre_len, suf_len, pre_off, suf_off, pre_seq, suf_seq;
     DevBuf smask, pmask;  // successor / predecessor bitsets (bitsets of <= MASK_MAX_W words)
+    DevBuf cmask, dflags, xinfo, dropD, dropX, drop_lvl;  // paths that cannot become PPs (DoomDev), same graphs
     GraphDev gd{};
 
     // enumeration workspace
@@ -425,9 +447,12 @@ struct tpg_cfg {
     DevBuf trace;
     std::vector<long long> h_trace;  // the last call's trace, LEVEL_TRACE_WORDS per level
     std::vector<LevelRec> h_levels;
+    long long *h_dropped = nullptr;  // room for max_levels counts behind the staged levels
+    long long last_nodes = 0, last_peak = 0;  // arena nodes of the last call, and of its largest level
     int *h_small = nullptr;  // pinned staging for small read-backs (16 KB, see HandlePool)
     void *h_lvl_stage = nullptr;  // pinned staging for level tables too large for h_small
     size_t h_lvl_bytes = 0;
+    std::vector<char> h_lvl_plain;  // its stand-in
 };
 
 // one training batch of the learned sizer: a copy of a handle's graph,
@@ -506,7 +531,7 @@ void destroy_cfg(tpg_cfg *g) {
     }
     DevBuf *all[] = {&g->rp, &g->col, &g->prp, &g->pcol, &g->vgraph, &g->vbase, &g->entry, &g->exitv,
                      &g->tbl_base, &g->dist, &g->pred, &g->pre_len, &g->suf_len, &g->pre_off, &g->suf_off,
-                     &g->smask, &g->pmask,
+                     &g->smask, &g->pmask, &g->cmask, &g->dflags, &g->xinfo, &g->dropD, &g->dropX, &g->drop_lvl,
                      &g->pre_seq, &g->suf_seq, &g->tfl[0], &g->tfl[1], &g->tvis[0], &g->tvis[1], &g->tcnt[0], &g->tcnt[1],
                      &g->levels, &g->agg, &g->ctl, &g->s_keys[0], &g->s_keys[1],
                      &g->s_refs[0], &g->s_refs[1], &g->s_len, &g->s_tmp, &g->s_i32[0], &g->s_i32[1],
@@ -562,6 +587,21 @@ int new_cfg(void *stream, tpg_cfg **out) {
     return TPG_OK;
 }
 
+// What the frontier drops and counts instead (nothing in a counting run, which
+// wants every path of every root; counted: also how many there are).
+DoomDev doom_dev(const tpg_cfg *g, bool counted) {
+    DoomDev d{};
+    if (g->W > MASK_MAX_W || g->root_counts) return d;
+    d.cmask = g->cmask.as<unsigned>();
+    d.flags = g->dflags.as<unsigned char>();
+    d.xinfo = g->xinfo.as<int2>();
+    if (counted) {
+        d.D = g->dropD.as<unsigned long long>();
+        d.X = g->dropX.as<unsigned>();
+    }
+    return d;
+}
+
 // Predecessor CSR, BFS tables and tour tables (everything after the union
 // CSR, vgraph/vbase and entry/exit are on the device).  validate: check the
 // CSR on the device first, TPG_EINVAL if it fails (a single graph whose
@@ -576,7 +616,7 @@ int preprocess(tpg_cfg *g, const std::vector<long long> &tbl_base_h, bool valida
     RC(ensure(g, g->prp, sizeof(int) * (g->N + 1)));
     RC(ensure(g, g->pcol, sizeof(int) * std::max<long long>(g->M, 1)));
     RC(ensure(g, g->tbl_base, sizeof(long long) * tbl_base_h.size()));
-    const long long tbl = tbl_base_h.back();
+    const long long tbl = g->tbl = tbl_base_h.back();
     RC(ensure(g, g->dist, sizeof(int) * std::max<long long>(tbl, 1)));
     RC(ensure(g, g->pred, sizeof(int) * std::max<long long>(tbl, 1)));
     RC(ensure(g, g->pre_len, sizeof(int) * g->N));
@@ -587,6 +627,12 @@ int preprocess(tpg_cfg *g, const std::vector<long long> &tbl_base_h, bool valida
     if (masks) {
         RC(ensure(g, g->smask, sizeof(unsigned) * (size_t)g->N * g->W));
         RC(ensure(g, g->pmask, sizeof(unsigned) * (size_t)g->N * g->W));
+        RC(ensure(g, g->cmask, sizeof(unsigned) * (size_t)g->N * g->W));
+        RC(ensure(g, g->dflags, (size_t)g->N));
+        RC(ensure(g, g->xinfo, sizeof(int2) * (size_t)g->N));
+        RC(ensure(g, g->dropD, sizeof(unsigned long long) * (size_t)doom_d_cells(tbl, g->N) + 16));
+        RC(ensure(g, g->dropX, sizeof(unsigned) * (size_t)doom_x_cells(tbl, g->G) + 16));
+        RC(ensure(g, g->drop_lvl, sizeof(unsigned long long) * g->max_levels + 16));
     }
     if (small) {
         const long long bound = (long long)g->N * (g->N + 1) / 2;
@@ -632,7 +678,7 @@ int preprocess(tpg_cfg *g, const std::vector<long long> &tbl_base_h, bool valida
         if (!validate) CK(cudaMemsetAsync(g->ctl.p, 0, sizeof(int), s));
         CK(preprocess_small(d, g->prp.as<int>(), g->pcol.as<int>(), g->tbl_base.as<long long>(), validate, entry,
                             exit, g->ctl.as<int>(), s, masks ? g->smask.as<unsigned>() : nullptr,
-                            masks ? g->pmask.as<unsigned>() : nullptr));
+                            masks ? g->pmask.as<unsigned>() : nullptr, doom_dev(g, false)));
         if (!validate) return TPG_OK;  // launch errors surfaced above; the next call's read-back sees the rest
         CK(cudaMemcpyAsync(g->h_small, g->ctl.p, sizeof(int), cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));
@@ -649,6 +695,7 @@ int preprocess(tpg_cfg *g, const std::vector<long long> &tbl_base_h, bool valida
                       g->s_i64[0].as<long long>(), s));
     if (masks) CK(build_vertex_masks(d, g->smask.as<unsigned>(), g->pmask.as<unsigned>(), nullptr, s));
     CK(bfs_all_pairs(d, s, nullptr, g->max_arcs));
+    if (masks) CK(doom_tables(d, doom_dev(g, false), s));
     CK(tour_lengths(d, g->s_tmp.as<long long>(), s));
     long long *h = (long long *)g->h_small;
     CK(cudaMemcpyAsync(h, d.pre_off + g->N, sizeof(long long), cudaMemcpyDeviceToHost, s));
@@ -780,8 +827,9 @@ int enumerate_levels(tpg_cfg *g) {
     RC(alloc_enumeration(g));
     RC(alloc_fixed_workspace(g));
     if (!enum_shape_supported(g->W, g->shape)) g->shape = default_enum_shape(g->W);
-    CK(cudaMemsetAsync(g->levels.p, 0, sizeof(LevelRec) * g->max_levels, s));
-    CK(cudaMemsetAsync(g->ctl.p, 0, CTL_BYTES, s));
+    const DoomDev dm = doom_dev(g, true);
+    unsigned long long *drop_lvl = g->drop_lvl.as<unsigned long long>();
+    CK(enum_reset(g->gd, dm, g->tbl, g->levels.as<LevelRec>(), g->max_levels, g->ctl.p, drop_lvl, s));
     int start_level = 1;
     int2 *next_override = nullptr;
     float total_ms = 0.f;
@@ -790,6 +838,7 @@ int enumerate_levels(tpg_cfg *g) {
         DevBuf &ppseg = g->pp_segs.back();
         EnumArgs a{};
         a.g = g->gd;
+        a.dm = dm;
         a.seg = seg.as<int2>();
         a.seg_cap = seg_nodes(seg);
         a.seg_place = a.seg + a.seg_cap;
@@ -832,12 +881,17 @@ int enumerate_levels(tpg_cfg *g) {
         g->stats.tile_items = g->shape.items;
         g->h_levels.resize(g->max_levels);
         const size_t lv_bytes = sizeof(LevelRec) * g->max_levels;
-        void *stage = level_stage(g, lv_bytes);
-        CK(cudaMemcpyAsync(stage ? stage : (void *)g->h_levels.data(), g->levels.p, lv_bytes, cudaMemcpyDeviceToHost,
-                           s));
+        const size_t drop_bytes = sizeof(long long) * g->max_levels;
+        char *stage = (char *)level_stage(g, lv_bytes + drop_bytes);
+        if (!stage) {  // no page-locked memory: an ordinary buffer
+            g->h_lvl_plain.resize(lv_bytes + drop_bytes);
+            stage = g->h_lvl_plain.data();
+        }
+        CK(cudaMemcpyAsync(stage, g->levels.p, lv_bytes, cudaMemcpyDeviceToHost, s));
         CK(cudaMemcpyAsync(g->h_small, g->ctl.p, 2 * sizeof(int), cudaMemcpyDeviceToHost, s));
+        g->h_dropped = (long long *)(stage + lv_bytes);
         CK(cudaStreamSynchronize(s));
-        if (stage) std::memcpy(g->h_levels.data(), stage, lv_bytes);
+        std::memcpy(g->h_levels.data(), stage, lv_bytes);
         float ms = 0.f;
         cudaEventElapsedTime(&ms, g->ev[0], g->ev[1]);
         total_ms += ms;
@@ -903,10 +957,56 @@ int enumerate_levels(tpg_cfg *g) {
     }
 }
 
+// The dropped paths of a finished enumeration are added up on a stream of
+// their own while the PPs are put in order: one block per graph that walks
+// down the path lengths, 20 us (24 vertices) to 90 us (120) that leave the
+// rest of the GPU idle.  The host has seen the enumeration end, so nothing has
+// to be waited for, and no way out of the call leaves it running.
+class DropCount {
+public:
+    explicit DropCount(tpg_cfg *g) : g_(g), dm_(doom_dev(g, true)) {}
+    cudaError_t start() {
+        if (!dm_.D) return cudaSuccess;
+        side_ = handle_pool().get_side(g_->device);
+        on_ = side_ ? side_ : g_->stream;
+        running_ = true;
+        return doom_count(g_->gd, dm_, g_->levels.as<LevelRec>(), g_->max_levels,
+                          g_->drop_lvl.as<unsigned long long>(), on_);
+    }
+    // ask for the counts / wait for them (null: none were counted)
+    cudaError_t fetch() {
+        if (!dm_.D) return cudaSuccess;
+        return cudaMemcpyAsync(g_->h_dropped, g_->drop_lvl.p, sizeof(long long) * g_->max_levels,
+                               cudaMemcpyDeviceToHost, on_);
+    }
+    cudaError_t finish(const long long **counts) {
+        *counts = dm_.D ? g_->h_dropped : nullptr;
+        return wait();
+    }
+    ~DropCount() { wait(); }
+    DropCount(const DropCount &) = delete;
+    DropCount &operator=(const DropCount &) = delete;
+
+private:
+    cudaError_t wait() {
+        if (!running_) return cudaSuccess;
+        running_ = false;
+        const cudaError_t e = cudaStreamSynchronize(on_);
+        if (side_) handle_pool().put_side(g_->device, side_);
+        return e;
+    }
+    tpg_cfg *g_;
+    DoomDev dm_;
+    cudaStream_t side_ = nullptr, on_ = nullptr;
+    bool running_ = false;
+};
+
 int run_prime_paths(tpg_cfg *g) {
     cudaStream_t s = g->stream;
     drop_cache(g);
     RC(enumerate_levels(g));
+    DropCount drops(g);
+    CK(drops.start());
     // level summary
     std::vector<int> pp_levels;
     long long P = 0, V = 0, nodes = 0, peak = 0;
@@ -923,10 +1023,9 @@ int run_prime_paths(tpg_cfg *g) {
             V += (long long)k * L.pp_count;
         }
     }
-    g->stats.simple_paths = nodes;
-    g->stats.levels = K;
+    g->last_nodes = nodes;
+    g->last_peak = peak;
     g->stats.pp_levels = (int)pp_levels.size();
-    g->stats.peak_level_nodes = peak;
     g->stats.prime_paths = P;
     g->stats.pp_vertices = V;
     g->stats.bitset_words = g->W;
@@ -986,8 +1085,22 @@ int run_prime_paths(tpg_cfg *g) {
         CK(cudaMemcpyAsync(gptr->p, h, 2 * sizeof(long long), cudaMemcpyHostToDevice, s));
     }
     CK(cudaEventRecord(g->ev[3], s));
+    CK(drops.fetch());
     CK(cudaStreamSynchronize(s));
+    const long long *dropped;
+    CK(drops.finish(&dropped));
     cudaEventElapsedTime(&g->stats.t_order_ms, g->ev[2], g->ev[3]);
+    // all simple paths: the arena's and those that were only counted
+    for (int k = 1; k < g->max_levels && dropped; ++k) {
+        const long long c = g->h_levels[k].count + dropped[k];
+        if (c >= (long long)MAX31) return TPG_ETOOBIG;
+        nodes += dropped[k];
+        peak = std::max(peak, c);
+        if (c > 0) K = std::max(K, k);
+    }
+    g->stats.simple_paths = nodes;
+    g->stats.levels = K;
+    g->stats.peak_level_nodes = peak;
     g->P = P;
     g->V = V;
     g->pp_valid = true;
@@ -1306,9 +1419,9 @@ int capture_plan(tpg_cfg *g) {
     }
     cudaStream_t s = g->stream ? g->stream : p.own_stream;
     // capacities: explicit ones win, otherwise the exact sizes of the last run
-    const bool have_run = g->pp_valid && g->stats.simple_paths > 0;
-    p.seg_cap = std::max<long long>(have_run ? g->stats.simple_paths : g->node_cap, g->N);
-    p.lvl_cap = round_frontier_cap(std::max<long long>(have_run ? g->stats.peak_level_nodes : g->lvl_cap, g->N));
+    const bool have_run = g->pp_valid && g->last_nodes > 0;
+    p.seg_cap = std::max<long long>(have_run ? g->last_nodes : g->node_cap, g->N);
+    p.lvl_cap = round_frontier_cap(std::max<long long>(have_run ? g->last_peak : g->lvl_cap, g->N));
     p.pp_cap = std::max<long long>(have_run ? g->stats.prime_paths : g->pp_cap, 1);
     p.P_cap = std::max<long long>(g->out_cap[0] ? g->out_cap[0] : g->stats.prime_paths, 1);
     p.V_cap = std::max<long long>(g->out_cap[1] ? g->out_cap[1] : g->stats.pp_vertices, 1);
@@ -1361,6 +1474,7 @@ int capture_plan(tpg_cfg *g) {
 
     EnumArgs a{};
     a.g = g->gd;
+    a.dm = doom_dev(g, false);
     a.seg = p.seg.as<int2>();
     a.seg_cap = p.seg_cap;
     a.seg_place = a.seg + a.seg_cap;
@@ -1437,8 +1551,7 @@ int capture_plan(tpg_cfg *g) {
     cudaError_t e = cudaSuccess;
     int grid = 0;
     do {
-        if ((e = cudaMemsetAsync(g->levels.p, 0, sizeof(LevelRec) * g->max_levels, s))) break;
-        if ((e = cudaMemsetAsync(g->ctl.p, 0, CTL_BYTES, s))) break;
+        if ((e = enum_reset(g->gd, a.dm, g->tbl, g->levels.as<LevelRec>(), g->max_levels, g->ctl.p, nullptr, s))) break;
         if ((e = cudaMemsetAsync(p.counts.p, 0, sizeof(GmCounts), s))) break;
         if ((e = launch_enumerate(a, g->shape, g->num_sms, s, &grid))) break;
         if ((e = gm_enqueue_pp(m, s))) break;

@@ -64,6 +64,28 @@ struct GraphDev {
 };
 constexpr int MASK_MAX_W = 8;
 
+// Paths that cannot become PPs (doomed.cu; graphs of at most MASK_MAX_W words).
+// A path that leaves the strongly connected component (SCC) of its first
+// vertex while a predecessor of that vertex is off the path can never take it
+// up (it would have to come back), nor close: no path that begins with it is
+// prime.  The frontier drops such an extension and only counts it.
+struct DoomDev {
+    const unsigned *cmask;        // [N][W] successors in another SCC (null: nothing is dropped)
+    const unsigned char *flags;   // [N] DOOM_* bits
+    const int2 *xinfo;            // [N] entry vertices: {offset, rows} of their counters, else {-1, 0}
+    unsigned long long *D;        // dropped extensions by length and last vertex, or null (not counted)
+    unsigned *X;                  // entry vertex x's counters, in a graph of n vertices: row j holds its dropped
+                                  // extensions of j + 1 vertices by last vertex, then its paths of j vertices
+};
+enum : unsigned {
+    DOOM_CYCLIC = 1,  // the vertex's SCC holds a cycle
+    DOOM_LEAVES = 2,  // it has successors in another SCC
+    DOOM_ENTRY = 4,   // its SCC holds a cycle and can be entered at it
+};
+// offsets of a graph of n vertices with first vertex vb and table base tb
+__host__ __device__ inline long long doom_d_base(long long tb, long long vb) { return tb + 2 * vb; }  // rows 0 .. n + 1
+__host__ __device__ inline long long doom_x_base(long long tb, long long gid) { return 2 * tb + 1024 * gid; }
+
 // ---------------------------------------------------------------------------
 // memory-model helpers (PTX ISA: ld/st .relaxed.gpu, %globaltimer)
 // ---------------------------------------------------------------------------

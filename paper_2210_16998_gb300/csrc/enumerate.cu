@@ -127,25 +127,57 @@ __device__ __forceinline__ void ext_mask(const GraphDev &g, int first, int last,
 }
 
 // eval_path with the vertex bitsets, for a path whose visited set is `vis`
-// (last vertex included): the count word holds the number of extending
-// successors (CNT_WIDE form); with none, the path is prime iff every
-// predecessor of its first vertex is on it (the last vertex is never one
-// here: an arc last -> first would be an extension).
+// (last vertex included): the count word (CNT_MASK_BITS form).  While a
+// predecessor of the first vertex is off the path, extensions into another
+// strongly connected component are dropped (DoomDev).  A path without any
+// extension is prime iff every predecessor of its first vertex is on it (the
+// last vertex is never one here: an arc last -> first would be an extension).
 template <int W>
-__device__ __forceinline__ unsigned eval_mask(const GraphDev &g, int k, int first, int last, int vb,
+__device__ __forceinline__ unsigned eval_mask(const GraphDev &g, const DoomDev &dm, int k, int first, int last, int vb,
                                               const unsigned (&vis)[W]) {
     if (k >= 2 && first == last) return CNT_PP;
-    unsigned m[W];
+    unsigned m[W], off = 0u, dropped = 0u, c = 0u;
     ext_mask<W>(g, first, last, vb, vis, m);
-    unsigned c = 0;
-#pragma unroll
-    for (int j = 0; j < W; ++j) c += __popc(m[j]);
-    if (c) return CNT_WIDE | c;
     const unsigned *pm = g.pmask + (long long)first * W;
 #pragma unroll
-    for (int j = 0; j < W; ++j)
-        if (__ldg(pm + j) & ~vis[j]) return 0u;
-    return CNT_PP;
+    for (int j = 0; j < W; ++j) off |= __ldg(pm + j) & ~vis[j];
+    if (off && dm.cmask) {
+#pragma unroll
+        for (int j = 0; j < W; ++j) {
+            const unsigned cm = __ldg(dm.cmask + (long long)last * W + j);
+            dropped |= m[j] & cm;
+            m[j] &= ~cm;
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < W; ++j) c += __popc(m[j]);
+    const unsigned entry = dm.D && (__ldg(dm.flags + first) & DOOM_ENTRY) ? CNT_ENTRY : 0u;
+    if (off) return c | entry | (dropped ? CNT_DOOM : 0u);
+    return c ? c | CNT_ON : CNT_ON | CNT_PP;  // (an entry vertex's predecessor outside is never on its paths)
+}
+
+template <bool MASK>
+__device__ __forceinline__ int children(unsigned cw) {
+    if constexpr (MASK) return (int)(cw & CNT_MASK_BITS);
+    else return cnt_children(cw);
+}
+
+// counters of path (first .. last) of k vertices whose graph starts at vb
+struct DoomAt {
+    unsigned long long *D;  // row k + 1
+    unsigned *X;            // row k of the first vertex's counters (null unless it is an entry vertex)
+    int n;
+};
+__device__ __forceinline__ DoomAt doom_at(const GraphDev &g, const DoomDev &dm, int k, int first, int vb) {
+    const int gid = g.vgraph ? __ldg(g.vgraph + first) : 0;
+    const int n = (g.vgraph ? __ldg(g.vbase + gid + 1) : g.N) - vb;
+    const long long tb = __ldg(g.tbl_base + gid);
+    const int xo = __ldg(&dm.xinfo[first].x);
+    DoomAt a;
+    a.n = n;
+    a.D = dm.D + doom_d_base(tb, vb) + (long long)(k + 1) * n;
+    a.X = xo >= 0 ? dm.X + doom_x_base(tb, gid) + xo + (long long)k * (n + 1) : nullptr;
+    return a;
 }
 
 // position of the (r+1)-th set bit of m (r = 0: the lowest); m has more than r set bits
@@ -226,9 +258,9 @@ __device__ __forceinline__ int enum_prologue(const EnumArgs &a) {
         for (int j = 0; j < PI; ++j) {
             if (lo + j < hi) {
                 vb[j] = g.vgraph ? __ldg(g.vbase + __ldg(g.vgraph + first[j])) : 0;
-                if constexpr (MASK) cw[j] = eval_mask<W>(g, k, first[j], last[j], vb[j], vis[j]);
+                if constexpr (MASK) cw[j] = eval_mask<W>(g, a.dm, k, first[j], last[j], vb[j], vis[j]);
                 else cw[j] = eval_path<W>(g, k, first[j], last[j], vb[j], vis[j], -1);
-                cp += ((unsigned long long)cnt_children(cw[j]) << 32) | (cw[j] >> 15);
+                cp += ((unsigned long long)children<MASK>(cw[j]) << 32) | (cw[j] >> 15);
             }
         }
         unsigned long long tot;
@@ -263,7 +295,25 @@ __device__ __forceinline__ int enum_prologue(const EnumArgs &a) {
             if (i >= hi) continue;
             if (lplace) lplace[i] = make_int2(pos_c, pos_p);
             if (cw[j] & CNT_PP) lpp[pos_p++] = i;
-            if (cnt_children(cw[j]) == 0) continue;
+            if constexpr (MASK) {
+                if (a.dm.D && (cw[j] & (CNT_ENTRY | CNT_DOOM))) {
+                    // paths of an entry vertex, and dropped extensions
+                    const DoomAt at = doom_at(g, a.dm, k, first[j], vb[j]);
+                    if (at.X) atomicAdd(at.X + at.n, 1u);
+                    if (cw[j] & CNT_DOOM) {
+                        unsigned m[W];
+                        ext_mask<W>(g, first[j], last[j], vb[j], vis[j], m);
+#pragma unroll
+                        for (int ww = 0; ww < W; ++ww)
+                            for (unsigned x = m[ww] & __ldg(a.dm.cmask + (long long)last[j] * W + ww); x; x &= x - 1) {
+                                const int y = 32 * ww + __ffs(x) - 1;
+                                atomicAdd(at.D + y, 1ull);
+                                if (at.X) atomicAdd(at.X + y, 1u);
+                            }
+                    }
+                }
+            }
+            if (children<MASK>(cw[j]) == 0) continue;
             auto child = [&](int w) {
                 const int bb = w - vb[j];
                 next[pos_c] = make_int2(w, i);
@@ -278,6 +328,10 @@ __device__ __forceinline__ int enum_prologue(const EnumArgs &a) {
             if constexpr (MASK) {
                 unsigned m[W];
                 ext_mask<W>(g, first[j], last[j], vb[j], vis[j], m);
+                if (cw[j] & CNT_DOOM) {
+#pragma unroll
+                    for (int ww = 0; ww < W; ++ww) m[ww] &= ~__ldg(a.dm.cmask + (long long)last[j] * W + ww);
+                }
 #pragma unroll
                 for (int ww = 0; ww < W; ++ww)
                     for (unsigned x = m[ww]; x; x &= x - 1) child(vb[j] + 32 * ww + __ffs(x) - 1);
@@ -449,10 +503,10 @@ __global__ void __launch_bounds__(BLOCK, W <= 8 ? 1024 / BLOCK : 1) enumerate_ke
                 for (int w = 0; w < W; ++w) vis[w] = __ldcg(in_vis + w * a.lvl_cap + i);
                 const int vb = g.vgraph ? __ldg(g.vbase + __ldg(g.vgraph + fl.x)) : 0;
                 unsigned cw;
-                if constexpr (MASK) cw = eval_mask<W>(g, k, fl.x, fl.y, vb, vis);
+                if constexpr (MASK) cw = eval_mask<W>(g, a.dm, k, fl.x, fl.y, vb, vis);
                 else cw = eval_path<W>(g, k, fl.x, fl.y, vb, vis, -1);
                 cnt[i] = (unsigned short)cw;
-                c_sum += cnt_children(cw);
+                c_sum += children<MASK>(cw);
                 p_sum += cw >> 15;
             }
 #pragma unroll
@@ -634,7 +688,7 @@ __global__ void __launch_bounds__(BLOCK, W <= 8 ? 1024 / BLOCK : 1) enumerate_ke
 #pragma unroll 4
                 for (int i = clo + lane; i < lo; i += 32) {
                     const unsigned w = __ldcg(in_cnt + i);
-                    sc += (unsigned)cnt_children(w);
+                    sc += (unsigned)children<MASK>(w);
                     sp += w >> 15;
                 }
                 pos_c += (int)__reduce_add_sync(0xffffffffu, sc);
@@ -696,7 +750,7 @@ __global__ void __launch_bounds__(BLOCK, W <= 8 ? 1024 / BLOCK : 1) enumerate_ke
 #pragma unroll
                 for (int j = 0; j < ITEMS; ++j) {
                     const int i = t0 + j * 32 + lane;
-                    const int nch = cnt_children(cw[j]);
+                    const int nch = children<MASK>(cw[j]);
                     const bool pp = (cw[j] & CNT_PP) != 0;
                     int x = nch;
 #pragma unroll
@@ -723,7 +777,7 @@ __global__ void __launch_bounds__(BLOCK, W <= 8 ? 1024 / BLOCK : 1) enumerate_ke
                     const int excl = x - nch;
                     if (lplace && i < hi) lplace[i] = make_int2(pos_c + excl, pos_p + __popc(ppm & lt_mask));
                     int vb_l = 0, e0_l = 0;
-                    if (nch > 0) {
+                    if (nch > 0 || (MASK && (cw[j] & CNT_DOOM))) {
                         vb_l = g.vgraph ? __ldg(g.vbase + __ldg(g.vgraph + first[j])) : 0;
                         if constexpr (!MASK) e0_l = __ldg(g.rp + last[j]);
                     }
@@ -732,8 +786,9 @@ __global__ void __launch_bounds__(BLOCK, W <= 8 ? 1024 / BLOCK : 1) enumerate_ke
                     // share of the next level's chunk counts
                     // fbm: the parent's first vertex as a W-word bitset (with
                     // the vertex bitsets; a successor equal to it closes a cycle)
+                    // pcw: the parent's count word (CNT_ON carries over to the child)
                     auto emit = [&](int w, int cpos, int pf, int pvb, const unsigned (&pvis)[W], int pi,
-                                    const unsigned (&fbm)[W]) {
+                                    const unsigned (&fbm)[W], unsigned pcw) {
                         const bool closes = (w == pf);
                         const int bb = w - pvb;
                         unsigned cvis[W];  // the child's visited set
@@ -749,23 +804,31 @@ __global__ void __launch_bounds__(BLOCK, W <= 8 ? 1024 / BLOCK : 1) enumerate_ke
                                 cp = 1u;
                             } else {
                                 const unsigned *sm = g.smask + (long long)w * W;
-                                unsigned c = 0u;
+                                unsigned c = 0u, on = pcw & CNT_ON, dropped = 0u;
 #pragma unroll
                                 for (int ww = 0; ww < W; ++ww) c += __popc(__ldg(sm + ww) & (~cvis[ww] | fbm[ww]));
-                                if (c) {
-                                    c2w = CNT_WIDE | c;
-                                    cc = c;
-                                    cp = 0u;
-                                } else {
-                                    // prime iff every predecessor of the first vertex is on it
-                                    const unsigned *pm = g.pmask + (long long)pf * W;
-                                    unsigned off = 0u;
+                                // the predecessors of the first vertex matter
+                                // to a leaf and where the SCC can be left
+                                if (!on) {
+                                    const bool leaves = a.dm.cmask && (__ldg(a.dm.flags + w) & DOOM_LEAVES);
+                                    if (c == 0u || leaves) {
+                                        const unsigned *pm = g.pmask + (long long)pf * W;
+                                        unsigned off = 0u;
 #pragma unroll
-                                    for (int ww = 0; ww < W; ++ww) off |= __ldg(pm + ww) & ~cvis[ww];
-                                    cp = off ? 0u : 1u;
-                                    c2w = off ? 0u : CNT_PP;
-                                    cc = 0u;
+                                        for (int ww = 0; ww < W; ++ww) off |= __ldg(pm + ww) & ~cvis[ww];
+                                        if (!off) {
+                                            on = CNT_ON;
+                                        } else if (leaves) {
+                                            const unsigned *cm = a.dm.cmask + (long long)w * W;
+#pragma unroll
+                                            for (int ww = 0; ww < W; ++ww)
+                                                dropped += __popc(__ldg(sm + ww) & ~cvis[ww] & __ldg(cm + ww));
+                                        }
+                                    }
                                 }
+                                cp = c == 0u && on ? 1u : 0u;
+                                cc = c - dropped;
+                                c2w = cc | on | (pcw & CNT_ENTRY) | (dropped ? CNT_DOOM : 0u) | (cp ? CNT_PP : 0u);
                             }
                         } else {
                             c2w = eval_path<W>(g, k + 1, pf, w, pvb, pvis, w);
@@ -818,13 +881,42 @@ __global__ void __launch_bounds__(BLOCK, W <= 8 ? 1024 / BLOCK : 1) enumerate_ke
                     unsigned fbm_l[W];  // this lane's parent's first vertex (lane-wise writing)
                     if constexpr (MASK) {
                         first_bits(first[j], vb_l, fbm_l);
-                        if (nch > 0) {
+                        if (nch > 0 || (cw[j] & CNT_DOOM)) {
                             const unsigned *sm = g.smask + (long long)last[j] * W;
 #pragma unroll
                             for (int ww = 0; ww < W; ++ww) xm[ww] = __ldg(sm + ww) & (~vis[j][ww] | fbm_l[ww]);
                         } else {
 #pragma unroll
                             for (int ww = 0; ww < W; ++ww) xm[ww] = 0u;
+                        }
+                        // dropped extensions leave the mask; they, and the
+                        // paths of entry vertices, are counted (lanes with
+                        // the same counter add once)
+                        const bool drops = (cw[j] & CNT_DOOM) != 0u;
+                        const bool entry = (cw[j] & CNT_ENTRY) != 0u;
+                        if (__any_sync(0xffffffffu, drops || entry)) {
+                            DoomAt at{nullptr, nullptr, 0};
+                            if (a.dm.D && (drops || entry))
+                                at = doom_at(g, a.dm, k, first[j],
+                                             g.vgraph ? __ldg(g.vbase + __ldg(g.vgraph + first[j])) : 0);
+                            if (a.dm.D) {
+                                const unsigned peers = __match_any_sync(0xffffffffu, entry ? first[j] : -1);
+                                if (entry && lane == __ffs(peers) - 1) atomicAdd(at.X + at.n, (unsigned)__popc(peers));
+                            }
+#pragma unroll
+                            for (int ww = 0; ww < W; ++ww) {
+                                unsigned x = drops ? xm[ww] & __ldg(a.dm.cmask + (long long)last[j] * W + ww) : 0u;
+                                xm[ww] &= ~x;
+                                while (a.dm.D && __any_sync(0xffffffffu, x != 0u)) {
+                                    const int y = 32 * ww + __ffs(x) - 1;
+                                    unsigned long long *cell = x ? at.D + y : nullptr;
+                                    const unsigned peers = __match_any_sync(0xffffffffu, (unsigned long long)cell);
+                                    if (x && lane == __ffs(peers) - 1)
+                                        atomicAdd(cell, (unsigned long long)__popc(peers));
+                                    if (x && entry) atomicAdd(at.X + y, 1u);
+                                    x &= x - 1;
+                                }
+                            }
                         }
                     }
                     const bool lanewise = TPG_ENUM_LANEWISE &&
@@ -843,7 +935,7 @@ __global__ void __launch_bounds__(BLOCK, W <= 8 ? 1024 / BLOCK : 1) enumerate_ke
                                         w = vb_l + 32 * ww + __ffs(xm[ww]) - 1;
                                         xm[ww] &= xm[ww] - 1;
                                     }
-                                if (w >= 0) emit(w, pos_c + excl + r, first[j], vb_l, vis[j], pi, fbm_l);
+                                if (w >= 0) emit(w, pos_c + excl + r, first[j], vb_l, vis[j], pi, fbm_l, cw[j]);
                             }
                         } else {
                             unsigned m = cw[j] & CNT_BITS;
@@ -853,7 +945,7 @@ __global__ void __launch_bounds__(BLOCK, W <= 8 ? 1024 / BLOCK : 1) enumerate_ke
                                     m &= m - 1;
                                     // (clamped: a wrong count word must not index past the arcs)
                                     const int w = __ldg(g.col + min((unsigned)(e0_l + sidx), (unsigned)(g.M - 1)));
-                                    emit(w, pos_c + excl + r, first[j], vb_l, vis[j], pi, fbm_l);
+                                    emit(w, pos_c + excl + r, first[j], vb_l, vis[j], pi, fbm_l, 0u);
                                 }
                             }
                         }
@@ -877,6 +969,7 @@ __global__ void __launch_bounds__(BLOCK, W <= 8 ? 1024 / BLOCK : 1) enumerate_ke
                                 unsigned pm[W];
 #pragma unroll
                                 for (int ww = 0; ww < W; ++ww) pm[ww] = __shfl_sync(0xffffffffu, xm[ww], p);
+                                const unsigned pword = __shfl_sync(0xffffffffu, cw[j], p);
                                 if (q >= tot) continue;
                                 // the rank-th extending successor of the parent
                                 int w = -1, rr = rank;
@@ -890,7 +983,7 @@ __global__ void __launch_bounds__(BLOCK, W <= 8 ? 1024 / BLOCK : 1) enumerate_ke
                                 }
                                 unsigned fbm[W];
                                 first_bits(pf, pvb, fbm);
-                                if (w >= 0) emit(w, pos_c + q, pf, pvb, pvis, pi, fbm);
+                                if (w >= 0) emit(w, pos_c + q, pf, pvb, pvis, pi, fbm, pword);
                                 continue;
                             }
                             const int pl = __shfl_sync(0xffffffffu, last[j], p);
@@ -915,7 +1008,7 @@ __global__ void __launch_bounds__(BLOCK, W <= 8 ? 1024 / BLOCK : 1) enumerate_ke
                                 }
                                 w = __ldg(g.col + (e < pe1 ? e : pe1 - 1));
                             }
-                            emit(w, pos_c + q, pf, pvb, pvis, pi, fbm_l);
+                            emit(w, pos_c + q, pf, pvb, pvis, pi, fbm_l, 0u);
                         }
                     }
                     if (pp) {

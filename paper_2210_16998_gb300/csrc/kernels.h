@@ -41,6 +41,14 @@ __host__ __device__ inline int cnt_children(unsigned cw) {
     return (cw & CNT_WIDE) ? (int)(cw & CNT_BITS) : __builtin_popcount(cw & CNT_BITS);
 #endif
 }
+// count word of a path that is evaluated with the vertex bitsets: bits 0-9
+// are the number of its children, CNT_ON says that every predecessor of its
+// first vertex is on it (it may be clear although they are), CNT_DOOM that it
+// has dropped extensions, CNT_ENTRY that its first vertex is a DOOM_ENTRY one
+constexpr unsigned CNT_MASK_BITS = 0x3ffu;
+constexpr unsigned CNT_ENTRY = 0x800u;
+constexpr unsigned CNT_ON = 0x1000u;
+constexpr unsigned CNT_DOOM = 0x2000u;
 // control block of a launch (err, stop_level, ...); the frontier's grid
 // barrier lives at CTL_BAR_OFFSET
 constexpr int CTL_BYTES = 1024;
@@ -49,6 +57,7 @@ constexpr int CTL_HANDOFF_OFFSET = 64;    // level a frontier launch's single-bl
 
 struct EnumArgs {
     GraphDev g;
+    DoomDev dm;
     int2 *seg;               // current arena segment (nodes {last, parent})
     long long seg_cap;
     int2 *seg_place;         // the segment's places, node i's at [i] (null: not kept; see place_pps)
@@ -109,6 +118,20 @@ long long scan_total_index(long long n);
 cudaError_t scan_i64_finish(const long long *in, long long *out, long long n, const long long *tmp, cudaStream_t s);
 // exclusive scan of int32 inputs into int64 outputs (out[n] = total)
 cudaError_t scan_i32_to_i64(const int *in, long long *out, long long n, long long *tmp, cudaStream_t s);
+
+// doomed.cu
+// tables of every graph (cmask, flags, xinfo), from the BFS tables
+cudaError_t doom_tables(const GraphDev &g, const DoomDev &dm, cudaStream_t s);
+inline long long doom_d_cells(long long tbl, long long N) { return tbl + 2 * N; }
+inline long long doom_x_cells(long long tbl, long long G) { return 2 * tbl + 1024 * G; }
+// zero before an enumeration: `levels` (level_bytes), `ctl` (CTL_BYTES) and,
+// if dm counts, its counters and level[max_levels]
+cudaError_t enum_reset(const GraphDev &g, const DoomDev &dm, long long tbl, LevelRec *levels, int max_levels, void *ctl,
+                       unsigned long long *level, cudaStream_t s);
+// the dropped paths of every length (level[], added to) after a finished
+// enumeration; D is used up
+cudaError_t doom_count(const GraphDev &g, const DoomDev &dm, const LevelRec *levels, int max_levels,
+                       unsigned long long *level, cudaStream_t s);
 
 // order.cu
 // canonical ordering of PP references across levels (ancestor-index merge)
@@ -242,10 +265,12 @@ cudaError_t bfs_all_pairs(const GraphDev &g, cudaStream_t s, const int *gate, lo
 // One graph of at most PREP_SMALL_N vertices: optional CSR validation (sets
 // ERR_INVAL in *err, which must be zero on entry, and skips the rest), the
 // predecessor CSR, tbl_base, the BFS tables and the tour tables in three
-// launches; g.pre_seq / g.suf_seq must hold N(N+1)/2 entries each.
+// launches; g.pre_seq / g.suf_seq must hold N(N+1)/2 entries each.  With masks
+// (at most 256 vertices), the masks and the tables of dm as well.
 constexpr int PREP_SMALL_N = 1024;
 cudaError_t preprocess_small(const GraphDev &g, int *prp, int *pcol, long long *tbl_base, bool validate, int entry,
-                             int exit, int *err, cudaStream_t s, unsigned *smask = nullptr, unsigned *pmask = nullptr);
+                             int exit, int *err, cudaStream_t s, unsigned *smask = nullptr, unsigned *pmask = nullptr,
+                             const DoomDev &dm = DoomDev{});
 // successor / predecessor bitsets of every vertex (GraphDev::smask, pmask),
 // W <= MASK_MAX_W; nothing is done while *gate is nonzero (gate optional)
 cudaError_t build_vertex_masks(const GraphDev &g, unsigned *smask, unsigned *pmask, const int *gate, cudaStream_t s);

@@ -3,6 +3,7 @@
 // predecessor tie-break, and the per-vertex tour tables path(entry -> v) and
 // path(v -> exit) used to assemble test paths.
 #include "common.cuh"
+#include "doom_dev.cuh"
 #include "kernels.h"
 
 namespace tpg {
@@ -368,9 +369,13 @@ cudaError_t build_vertex_masks(const GraphDev &g, unsigned *smask, unsigned *pma
 // stage_pred the N x N predecessor table is first copied to dynamic shared
 // memory, so the path walks read shared memory.
 __global__ void __launch_bounds__(PREP_BLOCK) tour_small_kernel(GraphDev g, const int *gate, int stage_pred,
-                                                                unsigned *smask, unsigned *pmask) {
+                                                                unsigned *smask, unsigned *pmask, DoomDev dm) {
     extern __shared__ int pred_s[];
     if (*gate) return;
+    if (blockIdx.x == 1) {  // (graphs with masks: at most 256 vertices)
+        doom_tables_block<PREP_BLOCK>(g, dm, 0);
+        return;
+    }
     const int N = g.N, tid = threadIdx.x;
     if (smask)
         for (int v = tid; v < N; v += PREP_BLOCK) vertex_masks(g, v, smask, pmask);
@@ -399,7 +404,7 @@ __global__ void __launch_bounds__(PREP_BLOCK) tour_small_kernel(GraphDev g, cons
 }
 
 cudaError_t preprocess_small(const GraphDev &g, int *prp, int *pcol, long long *tbl_base, bool validate, int entry,
-                             int exit, int *err, cudaStream_t s, unsigned *smask, unsigned *pmask) {
+                             int exit, int *err, cudaStream_t s, unsigned *smask, unsigned *pmask, const DoomDev &dm) {
     if (g.G != 1 || g.N > PREP_SMALL_N) return cudaErrorInvalidValue;
     prep_small_kernel<<<1, PREP_BLOCK, sizeof(int) * (g.N + 1), s>>>(g, prp, pcol, tbl_base, validate ? 1 : 0,
                                                                      entry, exit, err);
@@ -414,7 +419,7 @@ cudaError_t preprocess_small(const GraphDev &g, int *prp, int *pcol, long long *
                                       (int)TOUR_STAGE_BYTES)) != cudaSuccess)
             return e;
     }
-    tour_small_kernel<<<1, PREP_BLOCK, stage ? pred_bytes : 0, s>>>(g, err, stage, smask, pmask);
+    tour_small_kernel<<<dm.cmask ? 2 : 1, PREP_BLOCK, stage ? pred_bytes : 0, s>>>(g, err, stage, smask, pmask, dm);
     note_launch();
     return cudaGetLastError();
 }
