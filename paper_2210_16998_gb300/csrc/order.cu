@@ -199,7 +199,10 @@ cudaError_t graph_ptr_from_ids(const int *ids, long long n, int G, long long *pt
 // level, read while its parent links are followed up and its child links
 // down, and its first vertex's offset is the same sum with level k's number
 // taken k times.  No level waits for another: what bounds it are two dependent
-// chains of loads per PP (L2 latency), so it runs with as many warps as fit.
+// chains of loads per PP (a quarter of them L2 hits), so a step's three loads
+// are issued together and it runs with as many threads as an SM holds (4096
+// graphs, 14.4M PPs: 4, 6, 8 blocks per SM 1.89, 1.43, 1.33 ms; with a node's
+// place read after its parent link, at 6 blocks and a grid for 8, 2.88 ms).
 // Order + materialise, against a bottom-up and a top-down sweep over all nodes
 // with a grid barrier per level and sweep: 120-vertex CFG (15.0M nodes, 54
 // levels, 1.09M PPs) 1.053 -> 0.259 ms; 333 graphs (10.1M nodes, 0.42M PPs)
@@ -211,9 +214,9 @@ struct PlaceLevel {
     long long pp_before;  // PPs of the levels before this one
     int count, pp_count;
 };
-constexpr int PLACE_BLOCK = 256;
+constexpr int PLACE_BLOCK = 256, PLACE_BLOCKS_SM = 8;
 
-__global__ void __launch_bounds__(PLACE_BLOCK) place_pps_kernel(PlaceArgs a) {
+__global__ void __launch_bounds__(PLACE_BLOCK, PLACE_BLOCKS_SM) place_pps_kernel(PlaceArgs a) {
     extern __shared__ __align__(16) unsigned char place_smem[];
     __shared__ int s_L;
     PlaceLevel *lv = (PlaceLevel *)place_smem;  // [max_levels], level 0 unused
@@ -247,26 +250,36 @@ __global__ void __launch_bounds__(PLACE_BLOCK) place_pps_kernel(PlaceArgs a) {
             if (lv[mid].pp_before <= t) lo = mid;
             else hi = mid - 1;
         }
-        const int j = lo;
-        const int q = (int)(t - lv[j].pp_before), idx = lv[j].pp[q];
-        long long rank = q, off = (long long)q * j;
-        int up = idx, down = lv[j].place[idx].x, ku = j, kd = j + 1;
-        while (ku > 1 || kd <= L) {
-            if (ku > 1) {
-                up = lv[ku].nodes[up].y;
-                --ku;
-                const int before = lv[ku].place[up].y;
-                rank += before;
-                off += (long long)before * ku;
+        const int j = lo, idx = lv[j].pp[(int)(t - lv[j].pp_before)];
+        long long rank = 0, off = 0;
+        // ku: the level of `up`, whose place and parent load together; kd: that of `down`
+        int up = idx, down = 0, ku = j, kd = L + 1;
+        {
+            const int2 pl = lv[j].place[up];
+            if (j > 1) up = lv[j].nodes[up].y;
+            rank = pl.y;
+            off = (long long)pl.y * j;
+            down = pl.x;
+            ku = j - 1;
+            kd = j + 1;
+        }
+        while (ku >= 1 || kd <= L) {
+            int parent = 0;
+            int2 pu = make_int2(0, 0), pd = pu;
+            if (ku >= 1) {
+                pu = lv[ku].place[up];
+                if (ku > 1) parent = lv[ku].nodes[up].y;
             }
             if (kd <= L) {
-                int2 pl = make_int2(kd < L ? lv[kd + 1].count : 0, lv[kd].pp_count);  // past the level's end
-                if (down < lv[kd].count) pl = lv[kd].place[down];
-                rank += pl.y;
-                off += (long long)pl.y * kd;
-                down = pl.x;
-                ++kd;
+                if (down < lv[kd].count) pd = lv[kd].place[down];
+                else pd = make_int2(kd < L ? lv[kd + 1].count : 0, lv[kd].pp_count);  // past the level's end
             }
+            rank += pu.y + (long long)pd.y;
+            off += (long long)pu.y * ku + (long long)pd.y * kd;
+            up = parent;
+            down = pd.x;
+            --ku;
+            ++kd;
         }
         a.refs[rank] = ((long long)j << 32) | (unsigned)idx;
         a.off[rank] = off;
@@ -282,7 +295,8 @@ cudaError_t place_pps(const PlaceArgs &a, int num_sms, cudaStream_t s) {
         if (e != cudaSuccess) return e;
     }
     const long long need = (a.cap + PLACE_BLOCK - 1) / PLACE_BLOCK;
-    const long long grid = need < 1 ? 1 : need < 8ll * num_sms ? need : 8ll * num_sms;
+    const long long fit = (long long)PLACE_BLOCKS_SM * num_sms;
+    const long long grid = need < 1 ? 1 : need < fit ? need : fit;
     place_pps_kernel<<<(unsigned)grid, PLACE_BLOCK, smem, s>>>(a);
     note_launch();
     return cudaGetLastError();
