@@ -401,6 +401,8 @@ struct tpg_cfg {
     DevBuf rp, col, prp, pcol, vgraph, vbase, entry, exitv, tbl_base, dist, pred;
     DevBuf pre_len, suf_len, pre_off, suf_off, pre_seq, suf_seq;
     DevBuf smask, pmask;  // successor / predecessor bitsets (bitsets of <= MASK_MAX_W words)
+    DevBuf arc_slot, end_slot;  // where a TP can leave the entry's BFS tree (tree_slots_block)
+    DevBuf tp_subs, tp_slots;   // the TP ordering's tables
     DevBuf cmask, dflags, xinfo, dropD, dropX, drop_lvl;  // paths that cannot become PPs (DoomDev), same graphs
     GraphDev gd{};
 
@@ -432,8 +434,8 @@ struct tpg_cfg {
         cudaGraphExec_t exec = nullptr;
         cudaStream_t own_stream = nullptr;
         DevBuf seg, ppseg, tfl[2], tvis[2], tcnt[2];
-        DevBuf lvl_pp_off, refs[2], len, scan_tmp, pp_graph, tp_len, run_start, run_rank, tp_graph0,
-            run_base, nruns, bounds0, tp_off0, tp_vert0, perm[2], keep, keep_off, keep_rank, tp_graph, counts,
+        DevBuf lvl_pp_off, refs[2], len, scan_tmp, pp_graph, tp_len, tp_start, sub_rank, pos_sub, subs, slots,
+            tp_off0, perm[2], keep, keep_off, keep_rank, tp_graph, counts,
             key_off, key;
         Block *pp_off = nullptr, *pp_vert = nullptr, *pp_gptr = nullptr;
         Block *tp_off = nullptr, *tp_vert = nullptr, *tp_gptr = nullptr;
@@ -511,8 +513,8 @@ void release_plan(tpg_cfg *g) {
     p.exec = nullptr;
     DevBuf *all[] = {&p.seg, &p.ppseg, &p.tfl[0], &p.tfl[1], &p.tvis[0], &p.tvis[1], &p.tcnt[0], &p.tcnt[1], &p.lvl_pp_off,
                      &p.refs[0], &p.refs[1], &p.len, &p.scan_tmp, &p.pp_graph, &p.tp_len,
-                     &p.run_start, &p.run_rank, &p.tp_graph0, &p.run_base, &p.nruns, &p.bounds0, &p.tp_off0,
-                     &p.tp_vert0, &p.perm[0], &p.perm[1], &p.keep, &p.keep_off, &p.keep_rank, &p.tp_graph,
+                     &p.tp_start, &p.sub_rank, &p.pos_sub, &p.subs, &p.slots, &p.tp_off0,
+                     &p.perm[0], &p.perm[1], &p.keep, &p.keep_off, &p.keep_rank, &p.tp_graph,
                      &p.counts, &p.key_off, &p.key};
     for (DevBuf *b : all) release(g, *b);
     Block *bl[] = {p.pp_off, p.pp_vert, p.pp_gptr, p.tp_off, p.tp_vert, p.tp_gptr};
@@ -531,7 +533,7 @@ void destroy_cfg(tpg_cfg *g) {
     }
     DevBuf *all[] = {&g->rp, &g->col, &g->prp, &g->pcol, &g->vgraph, &g->vbase, &g->entry, &g->exitv,
                      &g->tbl_base, &g->dist, &g->pred, &g->pre_len, &g->suf_len, &g->pre_off, &g->suf_off,
-                     &g->smask, &g->pmask, &g->cmask, &g->dflags, &g->xinfo, &g->dropD, &g->dropX, &g->drop_lvl,
+                     &g->smask, &g->pmask, &g->arc_slot, &g->end_slot, &g->tp_subs, &g->tp_slots, &g->cmask, &g->dflags, &g->xinfo, &g->dropD, &g->dropX, &g->drop_lvl,
                      &g->pre_seq, &g->suf_seq, &g->tfl[0], &g->tfl[1], &g->tvis[0], &g->tvis[1], &g->tcnt[0], &g->tcnt[1],
                      &g->levels, &g->agg, &g->ctl, &g->s_keys[0], &g->s_keys[1],
                      &g->s_refs[0], &g->s_refs[1], &g->s_len, &g->s_tmp, &g->s_i32[0], &g->s_i32[1],
@@ -623,6 +625,8 @@ int preprocess(tpg_cfg *g, const std::vector<long long> &tbl_base_h, bool valida
     RC(ensure(g, g->suf_len, sizeof(int) * g->N));
     RC(ensure(g, g->pre_off, sizeof(long long) * (g->N + 1)));
     RC(ensure(g, g->suf_off, sizeof(long long) * (g->N + 1)));
+    RC(ensure(g, g->arc_slot, sizeof(int) * std::max<long long>(g->M, 1)));
+    RC(ensure(g, g->end_slot, sizeof(int) * g->G));
     const bool masks = g->W <= MASK_MAX_W;
     if (masks) {
         RC(ensure(g, g->smask, sizeof(unsigned) * (size_t)g->N * g->W));
@@ -677,8 +681,8 @@ int preprocess(tpg_cfg *g, const std::vector<long long> &tbl_base_h, bool valida
         d.suf_seq = g->suf_seq.as<int>();
         if (!validate) CK(cudaMemsetAsync(g->ctl.p, 0, sizeof(int), s));
         CK(preprocess_small(d, g->prp.as<int>(), g->pcol.as<int>(), g->tbl_base.as<long long>(), validate, entry,
-                            exit, g->ctl.as<int>(), s, masks ? g->smask.as<unsigned>() : nullptr,
-                            masks ? g->pmask.as<unsigned>() : nullptr, doom_dev(g, false)));
+                            exit, g->ctl.as<int>(), s, g->arc_slot.as<int>(), g->end_slot.as<int>(),
+                            masks ? g->smask.as<unsigned>() : nullptr, masks ? g->pmask.as<unsigned>() : nullptr, doom_dev(g, false)));
         if (!validate) return TPG_OK;  // launch errors surfaced above; the next call's read-back sees the rest
         CK(cudaMemcpyAsync(g->h_small, g->ctl.p, sizeof(int), cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));
@@ -696,6 +700,7 @@ int preprocess(tpg_cfg *g, const std::vector<long long> &tbl_base_h, bool valida
     if (masks) CK(build_vertex_masks(d, g->smask.as<unsigned>(), g->pmask.as<unsigned>(), nullptr, s));
     CK(bfs_all_pairs(d, s, nullptr, g->max_arcs));
     if (masks) CK(doom_tables(d, doom_dev(g, false), s));
+    CK(tree_slots(d, g->arc_slot.as<int>(), g->end_slot.as<int>(), s));
     CK(tour_lengths(d, g->s_tmp.as<long long>(), s));
     long long *h = (long long *)g->h_small;
     CK(cudaMemcpyAsync(h, d.pre_off + g->N, sizeof(long long), cudaMemcpyDeviceToHost, s));
@@ -1186,6 +1191,35 @@ int make_result(tpg_cfg *g, Block *off, Block *vert, Block *gptr, long long P, l
     return TPG_OK;
 }
 
+// The TP ordering's arrays for up to P TPs in up to `subs` sub-runs: carved
+// from two buffers of their own; perm, start, sub_rank, pos_sub and the keys
+// are the caller's.
+int tp_order_arrays(tpg_cfg *g, DevBuf &subs_buf, DevBuf &slots_buf, long long subs, TpOrder *o) {
+    const long long slots = g->M + g->N;
+    const size_t n = (size_t)subs + 2;
+    RC(ensure(g, subs_buf, n * (sizeof(longlong2) + sizeof(int4) + 2 * sizeof(long long) + sizeof(unsigned long long) +
+                                sizeof(int2))));
+    RC(ensure(g, slots_buf, sizeof(long long) * (2 * (size_t)slots + 2)));
+    o->g = g->gd;
+    o->arc_slot = g->arc_slot.as<int>();
+    o->end_slot = g->end_slot.as<int>();
+    char *p = subs_buf.as<char>();
+    auto take = [&](auto *&q, size_t bytes) {
+        q = (std::remove_reference_t<decltype(q)>)p;
+        p += bytes;
+    };
+    take(o->sub_dst, n * sizeof(longlong2));
+    take(o->sub_info, n * sizeof(int4));
+    take(o->sub_start, n * sizeof(long long));
+    take(o->bounds, n * sizeof(long long));
+    take(o->sub_at, n * sizeof(unsigned long long));
+    take(o->sub_slot, n * sizeof(int2));
+    o->slot_n = slots_buf.as<long long>();
+    o->max_k = (int *)(o->slot_n + slots);  // zeroed with the slots
+    o->slot_at = o->slot_n + slots + 1;
+    return TPG_OK;
+}
+
 // ---------------------------------------------------------------------------
 // test paths
 // ---------------------------------------------------------------------------
@@ -1218,47 +1252,36 @@ int run_test_paths(tpg_cfg *g, Block **o_off, Block **o_vert, Block **o_gptr, lo
         *oTV = 0;
         return TPG_OK;
     }
-    // lengths, run starts, graph ids
+    // lengths, and how many sorted runs there are
     RC(ensure(g, g->s_i64[0], sizeof(long long) * (P + 1)));   // tp_len
-    RC(ensure(g, g->s_i64[1], sizeof(long long) * (P + 1)));   // run_rank
-    RC(ensure(g, g->s_i32[0], sizeof(int) * (P + 1)));         // run_start
-    RC(ensure(g, g->s_i32[1], sizeof(int) * (P + 1)));         // tp_graph
-    RC(ensure(g, g->s_tmp, sizeof(long long) * scan_tmp_elems(P + 1)));
+    RC(ensure(g, g->s_tmp, sizeof(long long) * scan_tmp_elems(std::max<long long>(P, g->M + g->N) + 1)));
     RC(ensure(g, g->ctl, CTL_BYTES));
     CK(cudaEventRecord(g->ev[4], s));
-    CK(cudaMemsetAsync(g->ctl.p, 0, sizeof(int), s));
+    CK(cudaMemsetAsync(g->ctl.p, 0, 4 * sizeof(long long), s));  // error word, -, runs, graphs with PPs
     long long *tp_len = g->s_i64[0].as<long long>();
-    long long *run_rank = g->s_i64[1].as<long long>();
-    int *run_start = g->s_i32[0].as<int>();
-    int *tp_graph = g->s_i32[1].as<int>();
-    CK(tp_lengths(pp_off, g->pp_ends.as<int2>(), pp_graph, P, g->gd, tp_len, run_start, tp_graph, g->ctl.as<int>(),
-                  s));
+    CK(tp_lengths(pp_off, g->pp_ends.as<int2>(), pp_graph, P, g->gd, tp_len, g->ctl.as<int>(),
+                  g->ctl.as<unsigned long long>() + 2, s));
     Block *tp_off = block_new(g->fns, sizeof(long long) * (P + 1), s);
     if (!tp_off) return TPG_ENOMEM;
     int rc = TPG_OK;
     Block *tp_vert = nullptr, *f_off = nullptr, *f_vert = nullptr, *f_gptr = nullptr;
-    long long TV = 0, R = 0, T = 0, FTV = 0;
+    long long TV = 0, T = 0, FTV = 0;
     long long *h = (long long *)g->h_small;
     do {
-        // the TP vertex total first: the offsets and the runs are needed only
+        // the TP vertex total first: the offsets are needed only
         // when the TP list differs from the PP list
         long long *tmp = g->s_tmp.as<long long>();
         if (cuda_err(scan_i64_sums(tp_len, P, tmp, s))) { rc = TPG_ECUDA; break; }
         cudaMemcpyAsync(h, tmp + scan_total_index(P), sizeof(long long), cudaMemcpyDeviceToHost, s);
-        cudaMemcpyAsync(h + 2, g->ctl.p, sizeof(int), cudaMemcpyDeviceToHost, s);
+        cudaMemcpyAsync(h + 1, g->ctl.p, 4 * sizeof(long long), cudaMemcpyDeviceToHost, s);
         if (cudaStreamSynchronize(s) != cudaSuccess) { rc = TPG_ECUDA; break; }
         TV = h[0];
         g->last_tv0 = TV;
-        if (((int *)(h + 2))[0] & ERR_UNREACH) { rc = TPG_EUNREACH; break; }
-        if (TV != g->V) {
-            if (cuda_err(scan_i64_finish(tp_len, (long long *)tp_off->p, P, tmp, s)) ||
-                cuda_err(scan_i32_to_i64(run_start, run_rank, P, tmp, s))) {
-                rc = TPG_ECUDA;
-                break;
-            }
-            cudaMemcpyAsync(h + 1, run_rank + P, sizeof(long long), cudaMemcpyDeviceToHost, s);
-            if (cudaStreamSynchronize(s) != cudaSuccess) { rc = TPG_ECUDA; break; }
-            R = h[1];
+        if (((int *)(h + 1))[0] & ERR_UNREACH) { rc = TPG_EUNREACH; break; }
+        const long long runs = h[3], graphs_with_pp = h[4];
+        if (TV != g->V && cuda_err(scan_i64_finish(tp_len, (long long *)tp_off->p, P, tmp, s))) {
+            rc = TPG_ECUDA;
+            break;
         }
         if (TV == g->V) {
             // A TP is never shorter than its PP, so equal totals mean every
@@ -1276,16 +1299,7 @@ int run_test_paths(tpg_cfg *g, Block **o_off, Block **o_vert, Block **o_gptr, lo
             if (pp_to_tp && cuda_err(tp_index_map(nullptr, nullptr, nullptr, P, pp_to_tp, s))) rc = TPG_ECUDA;
             break;
         }
-        // graphs that own at least one PP: one sorted run each means no merge
-        long long graphs_with_pp = 1;
-        if (g->G > 1) {
-            std::vector<long long> gp(g->G + 1);
-            cudaMemcpyAsync(gp.data(), g->pp_gptr->p, sizeof(long long) * (g->G + 1), cudaMemcpyDeviceToHost, s);
-            if (cudaStreamSynchronize(s) != cudaSuccess) { rc = TPG_ECUDA; break; }
-            graphs_with_pp = 0;
-            for (int i = 0; i < g->G; ++i) graphs_with_pp += gp[i + 1] > gp[i];
-        }
-        if (R == graphs_with_pp) {
+        if (runs == graphs_with_pp) {
             // every graph's TPs form one run: sorted, and distinct PPs with a
             // common first vertex give distinct TPs, so nothing to dedup
             tp_vert = block_new(g->fns, sizeof(int) * std::max<long long>(TV, 1), s);
@@ -1309,56 +1323,69 @@ int run_test_paths(tpg_cfg *g, Block **o_off, Block **o_vert, Block **o_gptr, lo
             if (pp_to_tp && cuda_err(tp_index_map(nullptr, nullptr, nullptr, P, pp_to_tp, s))) rc = TPG_ECUDA;
             break;
         }
-        // merge rounds over the runs inside every graph (a graph has at most
-        // one run per vertex: one per first vertex of its PPs), comparing
-        // packed keys (8 or 16 bits per vertex; at most TV / vpw + P words)
-        const int kbits = g->maxn <= 255 ? 8 : 16;
-        const long long K_ub = TV / (64 / kbits) + P + 1;
-        if ((rc = ensure(g, g->s_i64[2], sizeof(long long) * (R + 2))) ||
-            (rc = ensure(g, g->s_i64[3], sizeof(long long) * (2 * (long long)g->G + 2))) ||
+        // the sub-runs and their places; with many TPs their number is read
+        // back, so that their tables are no larger than they have to be
+        TpOrder o{};
+        if ((rc = ensure(g, g->s_i32[0], sizeof(int) * (P + 1))) ||        // start, later keep
+            (rc = ensure(g, g->s_i64[1], sizeof(long long) * (P + 1))) ||  // sub_rank, later keep_off
+            (rc = ensure(g, g->s_i32[1], sizeof(int) * (P + 1))) ||        // pos_sub
             (rc = ensure(g, g->s_refs[0], sizeof(long long) * (P + 1))) ||
             (rc = ensure(g, g->s_refs[1], sizeof(long long) * (P + 1))) ||
             (rc = ensure(g, g->s_len, sizeof(long long) * (P + 1))) ||
-            (rc = ensure(g, g->tp_key_off, sizeof(long long) * (P + 1))) ||
+            (rc = ensure(g, g->tp_key_off, sizeof(long long) * (P + 1))))
+            break;
+        o.g = g->gd;
+        o.pp_off = pp_off;
+        o.pp_vert = pp_vert;
+        o.pp_graph = pp_graph;
+        o.arc_slot = g->arc_slot.as<int>();
+        o.end_slot = g->end_slot.as<int>();
+        o.start = g->s_i32[0].as<int>();
+        o.sub_rank = g->s_i64[1].as<long long>();
+        o.pos_sub = g->s_i32[1].as<int>();
+        o.perm[0] = g->s_refs[0].as<long long>();
+        o.perm[1] = g->s_refs[1].as<long long>();
+        if (cuda_err(tp_order_mark(o, P, s)) || cuda_err(scan_i32_to_i64(o.start, o.sub_rank, P, tmp, s))) {
+            rc = TPG_ECUDA;
+            break;
+        }
+        long long subs = P;
+        if (P > 1 << 18) {
+            cudaMemcpyAsync(h, o.sub_rank + P, sizeof(long long), cudaMemcpyDeviceToHost, s);
+            if (cudaStreamSynchronize(s) != cudaSuccess) { rc = TPG_ECUDA; break; }
+            subs = h[0];
+        }
+        // packed keys (8 or 16 bits per vertex; at most TV / vpw + P words)
+        const int kbits = g->maxn <= 255 ? 8 : 16;
+        const long long K_ub = TV / (64 / kbits) + P + 1;
+        if ((rc = tp_order_arrays(g, g->tp_subs, g->tp_slots, subs, &o)) ||
             (rc = ensure(g, g->tp_key, sizeof(unsigned long long) * K_ub)))
             break;
         long long *key_off = g->tp_key_off.as<long long>();
         unsigned long long *key = g->tp_key.as<unsigned long long>();
-        if (cuda_err(tp_key_lengths((const long long *)tp_off->p, P, kbits, g->s_len.as<long long>(), s)) ||
-            cuda_err(scan_i64(g->s_len.as<long long>(), key_off, P, g->s_tmp.as<long long>(), s)) ||
+        o.key_off = key_off;
+        o.key = key;
+        o.bits = kbits;
+        if (cuda_err(cudaMemsetAsync(o.slot_n, 0, sizeof(long long) * (g->M + g->N + 1), s)) ||
+            cuda_err(tp_order_list(o, P, subs, s)) || cuda_err(scan_i64(o.slot_n, o.slot_at, g->M + g->N, tmp, s)) ||
+            cuda_err(tp_order_place(o, P, subs, s)) ||
+            cuda_err(tp_key_lengths((const long long *)tp_off->p, P, kbits, g->s_len.as<long long>(), s)) ||
+            cuda_err(scan_i64(g->s_len.as<long long>(), key_off, P, tmp, s)) ||
             cuda_err(tp_write_keys_parts(pp_off, pp_vert, pp_graph, P, g->gd, (const long long *)tp_off->p, kbits,
-                                         key_off, key, s))) {
+                                         key_off, key, s)) ||
+            cuda_err(tp_order_merge(o, P, std::min<long long>(runs, g->maxn), s))) {
             rc = TPG_ECUDA;
             break;
         }
-        long long *bounds = g->s_i64[2].as<long long>();
-        long long *run_base = g->s_i64[3].as<long long>(), *nruns = run_base + g->G;
-        long long *perm[2] = {g->s_refs[0].as<long long>(), g->s_refs[1].as<long long>()};
-        const long long *tp_gptr = (const long long *)g->pp_gptr->p;  // TP i comes from PP i
-        if (cuda_err(tp_run_bounds(run_start, run_rank, P, R, bounds, s)) ||
-            cuda_err(tp_run_bases(tp_gptr, run_rank, g->G, run_base, nruns, s)) || cuda_err(tp_iota(perm[0], P, s))) {
-            rc = TPG_ECUDA;
-            break;
-        }
-        int cp = 0;
-        const int rounds = tp_merge_rounds(g->maxn);
-        for (int r = 0; r < rounds && rc == TPG_OK; ++r) {
-            if (cuda_err(tp_merge_graph_round_keys(perm[cp], perm[cp ^ 1], bounds, run_base, nruns, tp_gptr, g->G, r,
-                                                   P, key_off, key, s)))
-                rc = TPG_ECUDA;
-            cp ^= 1;
-        }
-        if (rc) break;
         // dedup + compaction
-        int *keep = g->s_i32[0].as<int>();                 // reuse run_start
+        const long long *perm = o.perm[0];
+        int *keep = g->s_i32[0].as<int>();                 // reuse start
         long long *keep_len = g->s_i64[0].as<long long>(); // reuse tp_len
-        long long *keep_off = g->s_i64[1].as<long long>(); // reuse run_rank
-        long long *keep_rank = perm[cp ^ 1];
-        if (cuda_err(tp_dedup_flags_keys(perm[cp], P, (const long long *)tp_off->p, key_off, key, tp_graph, keep_len,
-                                         keep, s)) ||
-            cuda_err(scan_i64(keep_len, keep_off, P, g->s_tmp.as<long long>(), s)) ||
-            cuda_err(scan_i32_to_i64(keep, keep_rank, P, g->s_tmp.as<long long>(), s)) ||
-            (pp_to_tp && cuda_err(tp_index_map(perm[cp], keep, keep_rank, P, pp_to_tp, s)))) {
+        long long *keep_off = g->s_i64[1].as<long long>(); // reuse sub_rank
+        long long *keep_rank = o.perm[1];
+        if (cuda_err(tp_order_flags(o, P, (const long long *)tp_off->p, keep_len, keep, s)) ||
+            cuda_err(scan_i64(keep_len, keep_off, P, tmp, s)) || cuda_err(scan_i32_to_i64(keep, keep_rank, P, tmp, s)) ||
+            (pp_to_tp && cuda_err(tp_index_map(perm, keep, keep_rank, P, pp_to_tp, s)))) {
             rc = TPG_ECUDA;
             break;
         }
@@ -1373,7 +1400,7 @@ int run_test_paths(tpg_cfg *g, Block **o_off, Block **o_vert, Block **o_gptr, lo
         if (!f_off || !f_vert || !f_gptr) { rc = TPG_ENOMEM; break; }
         if ((rc = ensure(g, g->s_i32[2], sizeof(int) * (T + 1)))) break;
         int *f_graph = g->s_i32[2].as<int>();
-        if (cuda_err(tp_assemble(perm[cp], keep, keep_rank, P, pp_off, pp_vert, pp_graph, g->gd,
+        if (cuda_err(tp_assemble(perm, keep, keep_rank, P, pp_off, pp_vert, pp_graph, g->gd,
                                  (const long long *)tp_off->p, keep_off, (long long *)f_off->p, (int *)f_vert->p, f_graph,
                                  s))) {
             rc = TPG_ECUDA;
@@ -1442,17 +1469,15 @@ int capture_plan(tpg_cfg *g) {
     }
     RC(ensure(g, p.lvl_pp_off, sizeof(long long) * (g->max_levels + 1)));
     RC(ensure(g, p.len, sizeof(long long) * Pc));
-    RC(ensure(g, p.scan_tmp, sizeof(long long) * gm_scan_tmp_elems(Pc + 1)));
+    RC(ensure(g, p.scan_tmp, sizeof(long long) * std::max(gm_scan_tmp_elems(Pc + 1), scan_tmp_elems(g->M + g->N + 1))));
     RC(ensure(g, p.pp_graph, sizeof(int) * Pc));
     RC(ensure(g, p.tp_len, sizeof(long long) * Pc));
-    RC(ensure(g, p.run_start, sizeof(int) * Pc));
-    RC(ensure(g, p.run_rank, sizeof(long long) * (Pc + 1)));
-    RC(ensure(g, p.tp_graph0, sizeof(int) * Pc));
-    RC(ensure(g, p.run_base, sizeof(long long) * g->G));
-    RC(ensure(g, p.nruns, sizeof(long long) * g->G));
-    RC(ensure(g, p.bounds0, sizeof(long long) * (Pc + 1)));
+    RC(ensure(g, p.tp_start, sizeof(int) * Pc));
+    RC(ensure(g, p.sub_rank, sizeof(long long) * (Pc + 1)));
+    RC(ensure(g, p.pos_sub, sizeof(int) * Pc));
+    TpOrder order{};
+    RC(tp_order_arrays(g, p.subs, p.slots, Pc, &order));
     RC(ensure(g, p.tp_off0, sizeof(long long) * (Pc + 1)));
-    RC(ensure(g, p.tp_vert0, 16));  // (the raw TP list is never written: TPs are assembled in sorted order)
     RC(ensure(g, p.keep, sizeof(int) * Pc));
     RC(ensure(g, p.keep_off, sizeof(long long) * (Pc + 1)));
     RC(ensure(g, p.keep_rank, sizeof(long long) * (Pc + 1)));
@@ -1512,10 +1537,7 @@ int capture_plan(tpg_cfg *g) {
     m.num_sms = g->num_sms;
     m.tp_rounds = gm_tp_rounds(g->maxn);
     m.lvl_pp_off = p.lvl_pp_off.as<long long>();
-    for (int b = 0; b < 2; ++b) {
-        m.refs[b] = p.refs[b].as<long long>();
-        m.perm[b] = p.perm[b].as<long long>();
-    }
+    for (int b = 0; b < 2; ++b) m.refs[b] = p.refs[b].as<long long>();
     m.len = p.len.as<long long>();
     m.scan_tmp = p.scan_tmp.as<long long>();
     m.pp_off = (long long *)p.pp_off->p;
@@ -1523,18 +1545,24 @@ int capture_plan(tpg_cfg *g) {
     m.pp_graph = p.pp_graph.as<int>();
     m.pp_gptr = (long long *)p.pp_gptr->p;
     m.tp_len = p.tp_len.as<long long>();
-    m.run_start = p.run_start.as<int>();
-    m.run_rank = p.run_rank.as<long long>();
-    m.tp_graph0 = p.tp_graph0.as<int>();
-    m.run_base = p.run_base.as<long long>();
-    m.nruns = p.nruns.as<long long>();
-    m.bounds0 = p.bounds0.as<long long>();
     m.tp_off0 = p.tp_off0.as<long long>();
-    m.tp_vert0 = p.tp_vert0.as<int>();
     m.key_off = p.key_off.as<long long>();
     m.key = p.key.as<unsigned long long>();
     m.K_cap = K_cap;
     m.key_bits = key_bits;
+    order.pp_off = m.pp_off;
+    order.pp_vert = m.pp_vert;
+    order.pp_graph = g->G > 1 ? m.pp_graph : nullptr;
+    order.start = p.tp_start.as<int>();
+    order.sub_rank = p.sub_rank.as<long long>();
+    order.pos_sub = p.pos_sub.as<int>();
+    order.perm[0] = p.perm[0].as<long long>();
+    order.perm[1] = p.perm[1].as<long long>();
+    order.key_off = m.key_off;
+    order.key = m.key;
+    order.bits = key_bits;
+    m.order = order;
+    m.slots = g->M + g->N;
     m.keep = p.keep.as<int>();
     m.keep_off = p.keep_off.as<long long>();
     m.keep_rank = p.keep_rank.as<long long>();
@@ -2283,7 +2311,8 @@ static int sort_paths(tpg_cfg *g, const long long *off, const int *vert, long lo
                       Block **o_off, Block **o_vert, long long *oT, long long *oTV) {
     cudaStream_t s = g->stream;
     long long *hs = (long long *)g->h_small;
-    DevBuf klen, koff, key, rrank, bounds, rbase, perm0, perm1, keep, keep_len, keep_off, keep_rank, ids, fgraph, tmp, gp;
+    DevBuf klen, koff, key, rrank, subs_buf, slots_buf, pos, perm0, perm1, keep, keep_len, keep_off, keep_rank, ids, fgraph,
+        tmp;
     Block *f_off = nullptr, *f_vert = nullptr;
     const int kbits = g->maxn <= 255 ? 8 : 16;
     const long long K_ub = V / (64 / kbits) + n + 1;
@@ -2292,18 +2321,14 @@ static int sort_paths(tpg_cfg *g, const long long *off, const int *vert, long lo
     do {
         if ((rc = ensure(g, klen, sizeof(long long) * (n + 1))) || (rc = ensure(g, koff, sizeof(long long) * (n + 1))) ||
             (rc = ensure(g, key, sizeof(unsigned long long) * K_ub)) || (rc = ensure(g, rrank, sizeof(long long) * (n + 1))) ||
-            (rc = ensure(g, bounds, sizeof(long long) * (n + 2))) || (rc = ensure(g, rbase, sizeof(long long) * 2)) ||
+            (rc = ensure(g, pos, sizeof(int) * n)) ||
             (rc = ensure(g, perm0, sizeof(long long) * n)) || (rc = ensure(g, perm1, sizeof(long long) * n)) ||
             (rc = ensure(g, keep, sizeof(int) * n)) || (rc = ensure(g, keep_len, sizeof(long long) * n)) ||
             (rc = ensure(g, keep_off, sizeof(long long) * (n + 1))) ||
             (rc = ensure(g, keep_rank, sizeof(long long) * (n + 1))) || (rc = ensure(g, ids, sizeof(int) * n)) ||
-            (rc = ensure(g, tmp, sizeof(long long) * scan_tmp_elems(n + 1))) || (rc = ensure(g, gp, sizeof(long long) * 2)))
+            (rc = ensure(g, tmp, sizeof(long long) * scan_tmp_elems(n + 1))))
             break;
-        hs[8] = 0;
-        hs[9] = n;
-        long long *perm[2] = {perm0.as<long long>(), perm1.as<long long>()};
-        if ((rc = cuda_err(cudaMemcpyAsync(gp.p, hs + 8, 2 * sizeof(long long), cudaMemcpyHostToDevice, s))) ||
-            (rc = cuda_err(cudaMemsetAsync(ids.p, 0, sizeof(int) * n, s))) ||
+        if ((rc = cuda_err(cudaMemsetAsync(ids.p, 0, sizeof(int) * n, s))) ||
             (rc = cuda_err(tp_key_lengths(off, n, kbits, klen.as<long long>(), s))) ||
             (rc = cuda_err(scan_i64(klen.as<long long>(), koff.as<long long>(), n, tmp.as<long long>(), s))) ||
             (rc = cuda_err(tp_write_keys(off, vert, n, kbits, koff.as<long long>(), key.as<unsigned long long>(), s))) ||
@@ -2312,22 +2337,17 @@ static int sort_paths(tpg_cfg *g, const long long *off, const int *vert, long lo
             (rc = cuda_err(cudaStreamSynchronize(s))))
             break;
         const long long R = hs[0];
-        long long *nruns = rbase.as<long long>() + 1;
-        if ((rc = cuda_err(tp_run_bounds(run_start, rrank.as<long long>(), n, R, bounds.as<long long>(), s))) ||
-            (rc = cuda_err(tp_run_bases(gp.as<long long>(), rrank.as<long long>(), 1, rbase.as<long long>(), nruns, s))) ||
-            (rc = cuda_err(tp_iota(perm[0], n, s))))
-            break;
-        int cp = 0;
-        const int rounds = tp_merge_rounds(R);
-        for (int r = 0; r < rounds && rc == TPG_OK; ++r) {
-            rc = cuda_err(tp_merge_graph_round_keys(perm[cp], perm[cp ^ 1], bounds.as<long long>(), rbase.as<long long>(),
-                                                    nruns, gp.as<long long>(), 1, r, n, koff.as<long long>(),
-                                                    key.as<unsigned long long>(), s));
-            cp ^= 1;
-        }
-        if (rc) break;
-        if ((rc = cuda_err(tp_dedup_flags_keys(perm[cp], n, off, koff.as<long long>(), key.as<unsigned long long>(),
-                                               ids.as<int>(), keep_len.as<long long>(), keep.as<int>(), s))) ||
+        TpOrder o{};
+        if ((rc = tp_order_arrays(g, subs_buf, slots_buf, R, &o))) break;
+        o.pos_sub = pos.as<int>();
+        o.perm[0] = perm0.as<long long>();
+        o.perm[1] = perm1.as<long long>();
+        o.key_off = koff.as<long long>();
+        o.key = key.as<unsigned long long>();
+        o.bits = kbits;
+        if ((rc = cuda_err(tp_order_plain(o, n, run_start, rrank.as<long long>(), R, s))) ||
+            (rc = cuda_err(tp_order_merge(o, n, R, s))) ||
+            (rc = cuda_err(tp_order_flags(o, n, off, keep_len.as<long long>(), keep.as<int>(), s))) ||
             (rc = cuda_err(scan_i64(keep_len.as<long long>(), keep_off.as<long long>(), n, tmp.as<long long>(), s))) ||
             (rc = cuda_err(scan_i32_to_i64(keep.as<int>(), keep_rank.as<long long>(), n, tmp.as<long long>(), s))) ||
             (rc = cuda_err(cudaMemcpyAsync(hs, keep_rank.as<long long>() + n, sizeof(long long), cudaMemcpyDeviceToHost, s))) ||
@@ -2341,7 +2361,7 @@ static int sort_paths(tpg_cfg *g, const long long *off, const int *vert, long lo
         if (!f_off || !f_vert) { rc = TPG_ENOMEM; break; }
         if ((rc = ensure(g, fgraph, sizeof(int) * std::max<long long>(T, 1)))) break;
         hs[2] = TV;
-        if ((rc = cuda_err(tp_gather(perm[cp], keep.as<int>(), keep_rank.as<long long>(), n, off, vert, ids.as<int>(),
+        if ((rc = cuda_err(tp_gather(o.perm[0], keep.as<int>(), keep_rank.as<long long>(), n, off, vert, ids.as<int>(),
                                      keep_off.as<long long>(), (long long *)f_off->p, (int *)f_vert->p, fgraph.as<int>(),
                                      s))) ||
             (rc = cuda_err(cudaMemcpyAsync((long long *)f_off->p + T, hs + 2, sizeof(long long), cudaMemcpyHostToDevice,
@@ -2350,8 +2370,8 @@ static int sort_paths(tpg_cfg *g, const long long *off, const int *vert, long lo
             break;
     } while (false);
     if (rc != TPG_OK) cudaStreamSynchronize(s);
-    for (DevBuf *b : {&klen, &koff, &key, &rrank, &bounds, &rbase, &perm0, &perm1, &keep, &keep_len, &keep_off,
-                      &keep_rank, &ids, &fgraph, &tmp, &gp})
+    for (DevBuf *b : {&klen, &koff, &key, &rrank, &subs_buf, &slots_buf, &pos, &perm0, &perm1, &keep, &keep_len, &keep_off,
+                      &keep_rank, &ids, &fgraph, &tmp})
         release(g, *b);
     if (rc) {
         block_unref(f_off);

@@ -17,35 +17,10 @@ namespace tpg {
 namespace {
 
 constexpr int GMB = 256;      // threads per block of the streaming kernels
-constexpr int GM_ITEMS = 4;   // outputs per thread of the PP merge
-#ifndef TPG_TPM_ITEMS
-#define TPG_TPM_ITEMS 4  // outputs per thread of a TP merge round
-#endif
-constexpr int TPM_ITEMS = TPG_TPM_ITEMS;  // outputs per thread of the TP run merge
 constexpr int GM_SCAN_ITEMS = 8;
 constexpr long long GM_SCAN_TILE = (long long)GMB * GM_SCAN_ITEMS;
 
 __device__ __forceinline__ long long clampc(long long v, long long cap) { return v < 0 ? 0 : (v > cap ? cap : v); }
-
-// largest k in [0, n] with a[k] <= x (a non-decreasing, a[0] <= x)
-__device__ __forceinline__ int slot_of(const long long *a, int n, long long x) {
-    int lo = 0, hi = n;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (a[mid] <= x) lo = mid;
-        else hi = mid - 1;
-    }
-    return lo;
-}
-
-__device__ __forceinline__ long long slot_of64(const long long *a, long long lo, long long hi, long long x) {
-    while (lo < hi) {
-        const long long mid = (lo + hi + 1) >> 1;
-        if (a[mid] <= x) lo = mid;
-        else hi = mid - 1;
-    }
-    return lo;
-}
 
 // ---------------------------------------------------------------------------
 // device-count scans
@@ -188,15 +163,7 @@ __global__ void __launch_bounds__(GMB) gm_tp_len(GmArgs a) {
         if (pl == 0 || sl == 0) atomicOr(&a.counts->flags, GM_UNREACH);
         else len = (long long)(pl - 1) + (o1 - o0) + (sl - 1);
         a.tp_len[i] = len;
-        const int vpw = 64 / a.key_bits;
-        a.len[i] = (len + vpw - 1) / vpw;
-        a.tp_graph0[i] = gid;
-        int start = 1;
-        if (i > 0) {
-            const int gprev = g.G > 1 ? a.pp_graph[i - 1] : 0;
-            start = (gprev != gid) || (a.pp_vert[a.pp_off[i - 1]] != a.pp_vert[o0]);
-        }
-        a.run_start[i] = start;
+        a.len[i] = key_words(len, a.key_bits);
     }
 }
 
@@ -211,27 +178,23 @@ __global__ void gm_tp_check(GmArgs a) {
         GmCounts *c = a.counts;
         c->TV0 = a.tp_off0[clampc(c->P, a.P_cap)];
         if (c->TV0 > a.TV0_cap || a.key_off[clampc(c->P, a.P_cap)] > a.K_cap) atomicOr(&c->flags, GM_OVF_TPV0);
-        c->R = a.run_rank[clampc(c->P, a.P_cap)];
     }
 }
 
-__global__ void __launch_bounds__(GMB) gm_run_bases(GmArgs a) {
-    const long long P = gm_P_tp(a);
-    const int G = a.g.G;
-    for (int g = blockIdx.x * GMB + threadIdx.x; g < G; g += gridDim.x * GMB) {
-        const long long s0 = P ? a.pp_gptr[g] : 0, s1 = P ? a.pp_gptr[g + 1] : 0;
-        a.run_base[g] = P ? a.run_rank[s0] : 0;
-        a.nruns[g] = P ? a.run_rank[s1] - a.run_rank[s0] : 0;
-    }
+__global__ void __launch_bounds__(GMB) gm_order_mark(GmArgs a) {
+    tp_mark_subs(a.order, gm_P_tp(a), blockIdx.x * (long long)GMB + threadIdx.x, gridDim.x * (long long)GMB);
 }
-
-__global__ void __launch_bounds__(GMB) gm_bounds0(GmArgs a) {
-    const long long P = gm_P_tp(a);
-    for (long long i = blockIdx.x * (long long)GMB + threadIdx.x; i < P; i += (long long)gridDim.x * GMB) {
-        if (a.run_start[i]) a.bounds0[a.run_rank[i]] = i;
-        a.perm[0][i] = i;
-    }
-    if (blockIdx.x == 0 && threadIdx.x == 0) a.bounds0[P ? a.counts->R : 0] = P;
+__global__ void __launch_bounds__(GMB) gm_order_list(GmArgs a) {
+    tp_list_subs(a.order, gm_P_tp(a), blockIdx.x * (long long)GMB + threadIdx.x, gridDim.x * (long long)GMB);
+}
+__global__ void __launch_bounds__(GMB) gm_order_count(GmArgs a) {
+    tp_count_subs(a.order, gm_P_tp(a), blockIdx.x * (long long)GMB + threadIdx.x, gridDim.x * (long long)GMB);
+}
+__global__ void __launch_bounds__(GMB) gm_order_place_subs(GmArgs a) {
+    tp_place_subs(a.order, gm_P_tp(a), blockIdx.x * (long long)GMB + threadIdx.x, gridDim.x * (long long)GMB);
+}
+__global__ void __launch_bounds__(GMB) gm_order_place(GmArgs a) {
+    tp_place(a.order, gm_P_tp(a), blockIdx.x * (long long)GMB + threadIdx.x, gridDim.x * (long long)GMB);
 }
 
 // TP vertex at position p of TP i: prefix, PP, suffix
@@ -280,55 +243,20 @@ __global__ void __launch_bounds__(GMB) gm_tp_write(GmArgs a) {
     }
 }
 
-// one round of pairwise run merging inside every graph (both runs of a merge
-// belong to one graph, so the comparisons read no graph ids)
-__global__ void __launch_bounds__(GMB) gm_tp_merge_round(GmArgs a, int r, int buf) {
+constexpr int GM_MERGE_ITEMS = 4;  // outputs per thread of a merge round
+__global__ void __launch_bounds__(GMB) gm_tp_merge_round(GmArgs a, int r) {
     const long long P = gm_P_tp(a);
-    const long long *pin = a.perm[buf];
-    long long *pout = a.perm[buf ^ 1];
-    const int G = a.g.G;
-    const long long nthreads = (long long)gridDim.x * GMB;
-    for (long long d0 = (blockIdx.x * (long long)GMB + threadIdx.x) * TPM_ITEMS; d0 < P; d0 += nthreads * TPM_ITEMS) {
-        long long a_hi = 0, b_hi = -1, i = 0, j = 0;
-        for (int t = 0; t < TPM_ITEMS; ++t) {
-            const long long d = d0 + t;
-            if (d >= P) break;
-            if (d >= b_hi) {
-                const int gg = G > 1 ? slot_of64(a.pp_gptr, 0, G, d) : 0;
-                const long long rb = a.run_base[gg], nr = a.nruns[gg];
-                const long long q0 = slot_of64(a.bounds0, rb, rb + nr - 1, d) - rb;
-                const long long m = q0 >> (r + 1);
-                const long long qa = m << (r + 1), qb = qa + (1ll << r), qe = (m + 1) << (r + 1);
-                const long long a_lo = a.bounds0[rb + qa];
-                a_hi = a.bounds0[rb + (qb < nr ? qb : nr)];
-                b_hi = a.bounds0[rb + (qe < nr ? qe : nr)];
-                const long long na = a_hi - a_lo, nb = b_hi - a_hi, diag = d - a_lo;
-                long long lo = diag > nb ? diag - nb : 0, hi = diag < na ? diag : na;
-                while (lo < hi) {
-                    const long long mid = (lo + hi) >> 1;
-                    if (key_cmp_same_graph(pin[a_lo + mid], pin[a_hi + diag - mid - 1], a.key_off, a.key) <= 0)
-                        lo = mid + 1;
-                    else
-                        hi = mid;
-                }
-                i = a_lo + lo;
-                j = a_hi + (diag - lo);
-            }
-            bool take_a;
-            if (i >= a_hi) take_a = false;
-            else if (j >= b_hi) take_a = true;
-            else take_a = key_cmp_same_graph(pin[i], pin[j], a.key_off, a.key) <= 0;
-            pout[d] = take_a ? pin[i++] : pin[j++];
-        }
-    }
+    if (P <= 0 || *a.order.max_k <= 1 << r) return;
+    const long long step = (long long)gridDim.x * GMB * GM_MERGE_ITEMS;
+    for (long long d0 = (blockIdx.x * (long long)GMB + threadIdx.x) * GM_MERGE_ITEMS; d0 < P; d0 += step)
+        tp_merge_items<GM_MERGE_ITEMS>(a.order, r, P, d0);
 }
 
-__global__ void __launch_bounds__(GMB) gm_tp_dedup(GmArgs a, int buf) {
+__global__ void __launch_bounds__(GMB) gm_tp_dedup(GmArgs a) {
     const long long P = gm_P_tp(a);
-    const long long *perm = a.perm[buf];
     for (long long i = blockIdx.x * (long long)GMB + threadIdx.x; i < P; i += (long long)gridDim.x * GMB) {
-        const long long x = perm[i];
-        const int k = (i == 0) || key_cmp(perm[i - 1], x, a.key_off, a.key, a.tp_graph0) != 0;
+        const long long x = a.order.perm[0][i];
+        const int k = tp_differs(a.order, i);
         a.keep[i] = k;
         a.tp_len[i] = k ? a.tp_off0[x + 1] - a.tp_off0[x] : 0;
     }
@@ -352,9 +280,9 @@ __device__ __forceinline__ long long gm_P_final(const GmArgs &a) {
 // The kept TPs in sorted order, each assembled from its parts (prefix path,
 // PP, suffix path) straight into its final place: the TP list is never
 // written in PP order.
-__global__ void __launch_bounds__(GMB) gm_tp_gather(GmArgs a, int buf) {
+__global__ void __launch_bounds__(GMB) gm_tp_gather(GmArgs a) {
     const long long P = gm_P_final(a);
-    const long long *perm = a.perm[buf];
+    const long long *perm = a.order.perm[0];
     const GraphDev &g = a.g;
     const int sub = threadIdx.x & (TP_LANES - 1);
     const long long ngroups = (long long)gridDim.x * (GMB / TP_LANES);
@@ -374,7 +302,7 @@ __global__ void __launch_bounds__(GMB) gm_tp_gather(GmArgs a, int buf) {
         const long long len = a.tp_off0[x + 1] - a.tp_off0[x], d0 = a.keep_off[i];
         for (long long p = sub; p < len; p += TP_LANES) a.tp_vert[d0 + p] = t.at(p);
         if (sub == 0) {
-            a.tp_graph[rk] = a.tp_graph0[x];
+            a.tp_graph[rk] = gid;
             a.tp_off[rk] = d0;
         }
     }
@@ -436,29 +364,31 @@ cudaError_t gm_enqueue_tp(const GmArgs &a, cudaStream_t s) {
     cudaError_t e;
     if ((e = gm_scan<long long>(a.tp_len, a.tp_off0, &a.counts->P, a.P_cap, a.scan_tmp, nullptr, a.num_sms, s)))
         return e;
-    if ((e = gm_scan<int>(a.run_start, a.run_rank, &a.counts->P, a.P_cap, a.scan_tmp, nullptr, a.num_sms, s)))
-        return e;
     if ((e = gm_scan<long long>(a.len, a.key_off, &a.counts->P, a.P_cap, a.scan_tmp, nullptr, a.num_sms, s)))
         return e;
     gm_tp_check<<<1, 32, 0, s>>>(a);
-    gm_run_bases<<<grid, GMB, 0, s>>>(a);
-    gm_bounds0<<<grid, GMB, 0, s>>>(a);
+    gm_order_mark<<<grid, GMB, 0, s>>>(a);
+    note_launch(2);
+    if ((e = gm_scan<int>(a.order.start, a.order.sub_rank, &a.counts->P, a.P_cap, a.scan_tmp, nullptr, a.num_sms, s)))
+        return e;
+    if ((e = cudaMemsetAsync(a.order.slot_n, 0, sizeof(long long) * (a.slots + 1), s))) return e;
+    gm_order_list<<<grid, GMB, 0, s>>>(a);
+    gm_order_count<<<grid, GMB, 0, s>>>(a);
+    note_launch(2);
+    if ((e = scan_i64(a.order.slot_n, a.order.slot_at, a.slots, a.scan_tmp, s))) return e;
+    gm_order_place_subs<<<grid, GMB, 0, s>>>(a);
+    gm_order_place<<<grid, GMB, 0, s>>>(a);
     gm_tp_write<<<grid, GMB, 0, s>>>(a);
-    note_launch(4);
-    int buf = 0;
-    for (int r = 0; r < a.tp_rounds; ++r) {
-        gm_tp_merge_round<<<grid, GMB, 0, s>>>(a, r, buf);
-        note_launch();
-        buf ^= 1;
-    }
-    gm_tp_dedup<<<grid, GMB, 0, s>>>(a, buf);
-    note_launch();
+    note_launch(3);
+    for (int r = 0; r < a.tp_rounds; ++r) gm_tp_merge_round<<<grid, GMB, 0, s>>>(a, r);
+    gm_tp_dedup<<<grid, GMB, 0, s>>>(a);
+    note_launch(a.tp_rounds + 1);
     if ((e = gm_scan<long long>(a.tp_len, a.keep_off, &a.counts->P, a.P_cap, a.scan_tmp, nullptr, a.num_sms, s)))
         return e;
     if ((e = gm_scan<int>(a.keep, a.keep_rank, &a.counts->P, a.P_cap, a.scan_tmp, nullptr, a.num_sms, s)))
         return e;
     gm_tp_totals<<<1, 32, 0, s>>>(a);
-    gm_tp_gather<<<grid, GMB, 0, s>>>(a, buf);
+    gm_tp_gather<<<grid, GMB, 0, s>>>(a);
     gm_graph_ptr<<<grid, GMB, 0, s>>>(a.tp_graph, &a.counts->T, a.P_cap, a.g.G, a.tp_gptr, a.counts,
                                       GM_ENUM_FAILED | GM_OVF_PP | GM_OVF_PPV | GM_UNREACH | GM_OVF_TPV0 | GM_OVF_TPV);
     note_launch(3);

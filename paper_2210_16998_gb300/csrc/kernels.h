@@ -5,6 +5,7 @@
 #include <atomic>
 
 #include "common.cuh"
+#include "tp_order_dev.cuh"
 
 namespace tpg {
 
@@ -177,7 +178,7 @@ enum : int {
 };
 static_assert(GM_TIMEOUT == 16, "flag bits must stay distinct");
 struct GmCounts {
-    long long P, V, TV0, R, T, TV;
+    long long P, V, TV0, T, TV;
     int flags;
     int pp_buf;  // which keys/refs buffer holds the ordered PPs
 };
@@ -197,18 +198,13 @@ struct GmArgs {
     int *pp_graph;          // [P_cap] (batches)
     long long *pp_gptr;     // [G+1]
     long long *tp_len;      // [P_cap]
-    int *run_start;         // [P_cap]
-    long long *run_rank;    // [P_cap+1]
-    int *tp_graph0;         // [P_cap]
-    long long *run_base, *nruns;  // [G]
-    long long *bounds0;     // [P_cap+1]
     long long *tp_off0;     // [P_cap+1]
-    int *tp_vert0;          // unused: TPs are assembled from their parts in sorted order
     long long *key_off;     // [P_cap+1] word offsets of the packed TP keys
     unsigned long long *key;  // [K_cap] packed TP keys
     long long K_cap;
     int key_bits;           // 8 (graphs of <= 255 vertices) or 16
-    long long *perm[2];     // [P_cap]
+    TpOrder order;          // the TPs' order (arrays for P_cap TPs)
+    long long slots;        // TP slots of all graphs
     int *keep;              // [P_cap]
     long long *keep_off, *keep_rank;  // [P_cap+1]
     long long *tp_off;      // [P_cap+1]
@@ -265,12 +261,13 @@ cudaError_t bfs_all_pairs(const GraphDev &g, cudaStream_t s, const int *gate, lo
 // One graph of at most PREP_SMALL_N vertices: optional CSR validation (sets
 // ERR_INVAL in *err, which must be zero on entry, and skips the rest), the
 // predecessor CSR, tbl_base, the BFS tables and the tour tables in three
-// launches; g.pre_seq / g.suf_seq must hold N(N+1)/2 entries each.  With masks
-// (at most 256 vertices), the masks and the tables of dm as well.
+// launches; g.pre_seq / g.suf_seq must hold N(N+1)/2 entries each.  The TP
+// slots (tree_slots_block) as well and, with masks (at most 256 vertices), the
+// masks and the tables of dm.
 constexpr int PREP_SMALL_N = 1024;
 cudaError_t preprocess_small(const GraphDev &g, int *prp, int *pcol, long long *tbl_base, bool validate, int entry,
-                             int exit, int *err, cudaStream_t s, unsigned *smask = nullptr, unsigned *pmask = nullptr,
-                             const DoomDev &dm = DoomDev{});
+                             int exit, int *err, cudaStream_t s, int *arc_slot, int *end_slot, unsigned *smask = nullptr,
+                             unsigned *pmask = nullptr, const DoomDev &dm = DoomDev{});
 // successor / predecessor bitsets of every vertex (GraphDev::smask, pmask),
 // W <= MASK_MAX_W; nothing is done while *gate is nonzero (gate optional)
 cudaError_t build_vertex_masks(const GraphDev &g, unsigned *smask, unsigned *pmask, const int *gate, cudaStream_t s);
@@ -279,12 +276,9 @@ cudaError_t tour_fill(const GraphDev &g, cudaStream_t s);
 
 // testpaths.cu
 cudaError_t tp_lengths(const long long *pp_off, const int2 *pp_ends, const int *pp_graph, long long P,
-                       const GraphDev &g, long long *tp_len, int *run_start, int *tp_graph, int *err,
-                       cudaStream_t s);
+                       const GraphDev &g, long long *tp_len, int *err, unsigned long long *runs, cudaStream_t s);
 cudaError_t tp_write(const long long *pp_off, const int *pp_vert, const int *pp_graph, long long P,
                      const GraphDev &g, const long long *tp_off, int *tp_vert, cudaStream_t s);
-cudaError_t tp_run_bounds(const int *run_start, const long long *run_rank, long long P, long long R,
-                          long long *bounds, cudaStream_t s);
 cudaError_t tp_iota(long long *perm, long long P, cudaStream_t s);
 cudaError_t tp_gather(const long long *perm, const int *keep, const long long *keep_rank, long long P,
                       const long long *tp_off, const int *tp_vert, const int *tp_graph,

@@ -6,29 +6,21 @@ namespace tpg {
 
 // Packed comparison keys of vertex sequences: vertex v is stored as v + 1
 // in `bits` (8 or 16) bits, most significant first, vpw = 64 / bits vertices
-// per 64-bit word, the last word zero-padded.  Comparing word by word (a
-// missing word reads as 0) orders the sequences lexicographically with a
-// proper prefix first, and equal keys mean equal sequences.  This form
-// compares two sequences of the same graph (no graph ids read); key_cmp
-// orders by graph id first.
-__device__ __forceinline__ int key_cmp_same_graph(long long a, long long b, const long long *koff,
-                                                  const unsigned long long *key) {
-    const long long a0 = koff[a], wa = koff[a + 1] - a0;
-    const long long b0 = koff[b], wb = koff[b + 1] - b0;
-    const long long w = wa > wb ? wa : wb;
-    for (long long t = 0; t < w; ++t) {
-        const unsigned long long x = t < wa ? key[a0 + t] : 0ull;
-        const unsigned long long y = t < wb ? key[b0 + t] : 0ull;
-        if (x != y) return x < y ? -1 : 1;
-    }
-    return 0;
+// per 64-bit word; a sequence of len vertices takes len / vpw + 1 words, so its
+// last word ends in zero bits (key_end) and no length is needed to compare.
+// Comparing word by word orders the sequences lexicographically with a proper
+// prefix first, and equal keys mean equal sequences.
+__host__ __device__ inline long long key_words(long long len, int bits) { return len / (64 / bits) + 1; }
+__device__ __forceinline__ bool key_end(unsigned long long word, int bits) {
+    return (word & ((1ull << bits) - 1)) == 0ull;
 }
 
-__device__ __forceinline__ int key_cmp(long long a, long long b, const long long *koff,
-                                       const unsigned long long *key, const int *graph) {
-    const int ga = graph[a], gb = graph[b];
-    if (ga != gb) return ga < gb ? -1 : 1;
-    return key_cmp_same_graph(a, b, koff, key);
+__device__ __forceinline__ int key_cmp_words(const unsigned long long *a, const unsigned long long *b, int bits) {
+    for (;; ++a, ++b) {
+        const unsigned long long x = *a, y = *b;
+        if (x != y) return x < y ? -1 : 1;
+        if (key_end(x, bits)) return 0;
+    }
 }
 
 // Materialise PPs [0, n): one warp handles 32 * CH consecutive PPs, CH per

@@ -5,6 +5,7 @@
 #include "common.cuh"
 #include "doom_dev.cuh"
 #include "kernels.h"
+#include "tp_order_dev.cuh"
 
 namespace tpg {
 
@@ -369,10 +370,15 @@ cudaError_t build_vertex_masks(const GraphDev &g, unsigned *smask, unsigned *pma
 // stage_pred the N x N predecessor table is first copied to dynamic shared
 // memory, so the path walks read shared memory.
 __global__ void __launch_bounds__(PREP_BLOCK) tour_small_kernel(GraphDev g, const int *gate, int stage_pred,
-                                                                unsigned *smask, unsigned *pmask, DoomDev dm) {
+                                                                int *arc_slot, int *end_slot, unsigned *smask,
+                                                                unsigned *pmask, DoomDev dm) {
     extern __shared__ int pred_s[];
     if (*gate) return;
-    if (blockIdx.x == 1) {  // (graphs with masks: at most 256 vertices)
+    if (blockIdx.x == 1) {
+        tree_slots_block<PREP_BLOCK>(g, 0, arc_slot, end_slot, pred_s);
+        return;
+    }
+    if (blockIdx.x == 2) {  // (graphs with masks: at most 256 vertices)
         doom_tables_block<PREP_BLOCK>(g, dm, 0);
         return;
     }
@@ -404,7 +410,8 @@ __global__ void __launch_bounds__(PREP_BLOCK) tour_small_kernel(GraphDev g, cons
 }
 
 cudaError_t preprocess_small(const GraphDev &g, int *prp, int *pcol, long long *tbl_base, bool validate, int entry,
-                             int exit, int *err, cudaStream_t s, unsigned *smask, unsigned *pmask, const DoomDev &dm) {
+                             int exit, int *err, cudaStream_t s, int *arc_slot, int *end_slot, unsigned *smask,
+                             unsigned *pmask, const DoomDev &dm) {
     if (g.G != 1 || g.N > PREP_SMALL_N) return cudaErrorInvalidValue;
     prep_small_kernel<<<1, PREP_BLOCK, sizeof(int) * (g.N + 1), s>>>(g, prp, pcol, tbl_base, validate ? 1 : 0,
                                                                      entry, exit, err);
@@ -414,12 +421,14 @@ cudaError_t preprocess_small(const GraphDev &g, int *prp, int *pcol, long long *
     if ((e = bfs_all_pairs(g, s, err, g.M)) != cudaSuccess) return e;
     const size_t pred_bytes = sizeof(int) * (size_t)g.N * g.N;
     const int stage = pred_bytes <= TOUR_STAGE_BYTES;
-    if (stage && pred_bytes > 48 * 1024) {
+    if (stage && pred_bytes > 32 * 1024) {  // (with the kernel's own arrays more than 48 KB)
         if ((e = cudaFuncSetAttribute(tour_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)TOUR_STAGE_BYTES)) != cudaSuccess)
             return e;
     }
-    tour_small_kernel<<<dm.cmask ? 2 : 1, PREP_BLOCK, stage ? pred_bytes : 0, s>>>(g, err, stage, smask, pmask, dm);
+    const size_t slot_bytes = 3 * sizeof(int) * (size_t)g.N;
+    tour_small_kernel<<<dm.cmask ? 3 : 2, PREP_BLOCK, stage && pred_bytes > slot_bytes ? pred_bytes : slot_bytes, s>>>(
+        g, err, stage, arc_slot, end_slot, smask, pmask, dm);
     note_launch();
     return cudaGetLastError();
 }

@@ -5,12 +5,9 @@
 // at the shared endpoints (Problem 1 output; the touring of Sec. 7.3), with
 // path(a -> b) read from the lowest-id BFS predecessor table.  Because the
 // PPs arrive in canonical order, TPs of PPs that share a first vertex share
-// their prefix and are already in order among themselves; so the TP list is
-// a sequence of sorted runs (one per (graph, first vertex)).  The runs of
-// each graph are merged pairwise (merge path) in ceil(log2(runs)) rounds,
-// comparing packed keys (8 or 16 bits per vertex, 64-bit words), and exact
-// duplicates (two PPs of different first vertices can yield the same TP)
-// are dropped after the final round.
+// their prefix and are already in order among themselves.  How the whole list
+// is put in order is told in tp_order_dev.cuh; exact duplicates (two PPs of
+// different first vertices can yield the same TP) are dropped at the end.
 #include "common.cuh"
 #include "kernels.h"
 #include "paths_dev.cuh"
@@ -25,13 +22,15 @@ static unsigned grid_for(long long n, int block = 256) {
     return (unsigned)b;
 }
 
-// TP lengths and run starts from each PP's (first, last) local vertex, which
-// the materialisation wrote beside the PP list (coalesced reads only).
-__global__ void tp_len_kernel(const long long *__restrict__ pp_off, const int2 *__restrict__ pp_ends,
-                              const int *__restrict__ pp_graph, long long P, GraphDev g, long long *tp_len,
-                              int *run_start, int *tp_graph, int *err) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < P;
-         i += (long long)gridDim.x * blockDim.x) {
+// TP lengths from each PP's (first, last) local vertex, which the
+// materialisation wrote beside the PP list (coalesced reads only); runs[0] +=
+// runs of PPs with one first vertex, runs[1] += graphs that own a PP.
+__global__ void __launch_bounds__(256) tp_len_kernel(const long long *__restrict__ pp_off,
+                                                     const int2 *__restrict__ pp_ends,
+                                                     const int *__restrict__ pp_graph, long long P, GraphDev g,
+                                                     long long *tp_len, int *err, unsigned long long *runs) {
+    int nruns = 0, ngraphs = 0;
+    for (long long i = blockIdx.x * 256ll + threadIdx.x; i < P; i += gridDim.x * 256ll) {
         const long long o0 = pp_off[i], o1 = pp_off[i + 1];
         const int gid = pp_graph ? pp_graph[i] : 0;
         const int vb = g.vgraph ? g.vbase[gid] : 0;
@@ -42,21 +41,23 @@ __global__ void tp_len_kernel(const long long *__restrict__ pp_off, const int2 *
         if (pl == 0 || sl == 0) atomicOr(err, ERR_UNREACH);
         else len = (long long)(pl - 1) + (o1 - o0) + (sl - 1);
         tp_len[i] = len;
-        tp_graph[i] = gid;
-        int start = 1;
-        if (i > 0) {
-            const int gprev = pp_graph ? pp_graph[i - 1] : 0;
-            start = (gprev != gid) || (pp_ends[i - 1].x != e.x);
-        }
-        run_start[i] = start;
+        const bool new_graph = i == 0 || (pp_graph && pp_graph[i - 1] != gid);
+        ngraphs += new_graph;
+        nruns += new_graph || pp_ends[i - 1].x != e.x;
+    }
+    nruns = __reduce_add_sync(0xffffffffu, nruns);
+    ngraphs = __reduce_add_sync(0xffffffffu, ngraphs);
+    if ((threadIdx.x & 31) == 0 && nruns) {
+        atomicAdd(runs, (unsigned long long)nruns);
+        if (ngraphs) atomicAdd(runs + 1, (unsigned long long)ngraphs);
     }
 }
 
 cudaError_t tp_lengths(const long long *pp_off, const int2 *pp_ends, const int *pp_graph, long long P,
-                       const GraphDev &g, long long *tp_len, int *run_start, int *tp_graph, int *err,
-                       cudaStream_t s) {
+                       const GraphDev &g, long long *tp_len, int *err, unsigned long long *runs, cudaStream_t s) {
     if (P <= 0) return cudaSuccess;
-    tp_len_kernel<<<grid_for(P), 256, 0, s>>>(pp_off, pp_ends, pp_graph, P, g, tp_len, run_start, tp_graph, err);
+    const unsigned grid = grid_for(P);
+    tp_len_kernel<<<grid < 4864 ? grid : 4864, 256, 0, s>>>(pp_off, pp_ends, pp_graph, P, g, tp_len, err, runs);
     note_launch();
     return cudaGetLastError();
 }
@@ -136,26 +137,13 @@ cudaError_t tp_write(const long long *pp_off, const int *pp_vert, const int *pp_
     return cudaGetLastError();
 }
 
-__global__ void run_bounds_kernel(const int *run_start, const long long *run_rank, long long P, long long R,
-                                  long long *bounds) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < P;
-         i += (long long)gridDim.x * blockDim.x)
-        if (run_start[i]) bounds[run_rank[i]] = i;
-    if (blockIdx.x == 0 && threadIdx.x == 0) bounds[R] = P;
-}
-
-cudaError_t tp_run_bounds(const int *run_start, const long long *run_rank, long long P, long long R,
-                          long long *bounds, cudaStream_t s) {
-    run_bounds_kernel<<<grid_for(P), 256, 0, s>>>(run_start, run_rank, P, R, bounds);
-    note_launch();
-    return cudaGetLastError();
-}
-
 __global__ void iota_kernel(long long *perm, long long P) {
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < P;
          i += (long long)gridDim.x * blockDim.x)
         perm[i] = i;
 }
+
+
 
 cudaError_t tp_iota(long long *perm, long long P, cudaStream_t s) {
     if (P <= 0) return cudaSuccess;
@@ -164,114 +152,124 @@ cudaError_t tp_iota(long long *perm, long long P, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-#ifndef TPG_TPM_ITEMS
-#define TPG_TPM_ITEMS 4  // outputs per thread of a TP merge round
-#endif
-constexpr int TPM_ITEMS = TPG_TPM_ITEMS;
-
-// largest s in [lo, hi] with a[s] <= x (a nondecreasing, a[lo] <= x)
-__device__ __forceinline__ long long tp_slot(const long long *a, long long lo, long long hi, long long x) {
-    while (lo < hi) {
-        const long long mid = (lo + hi + 1) >> 1;
-        if (a[mid] <= x) lo = mid;
-        else hi = mid - 1;
-    }
-    return lo;
+__global__ void __launch_bounds__(256) tp_mark_kernel(TpOrder o, long long P) {
+    tp_mark_subs(o, P, blockIdx.x * 256ll + threadIdx.x, gridDim.x * 256ll);
+}
+__global__ void __launch_bounds__(256) tp_list_kernel(TpOrder o, long long P) {
+    tp_list_subs(o, P, blockIdx.x * 256ll + threadIdx.x, gridDim.x * 256ll);
+}
+__global__ void __launch_bounds__(256) tp_count_kernel(TpOrder o, long long P) {
+    tp_count_subs(o, P, blockIdx.x * 256ll + threadIdx.x, gridDim.x * 256ll);
+}
+__global__ void __launch_bounds__(256) tp_place_subs_kernel(TpOrder o, long long P) {
+    tp_place_subs(o, P, blockIdx.x * 256ll + threadIdx.x, gridDim.x * 256ll);
+}
+__global__ void __launch_bounds__(256) tp_place_kernel(TpOrder o, long long P) {
+    tp_place(o, P, blockIdx.x * 256ll + threadIdx.x, gridDim.x * 256ll);
 }
 
-__global__ void run_bases_kernel(const long long *gptr, const long long *run_rank, int G, long long *run_base,
-                                 long long *nruns) {
-    for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < G; g += gridDim.x * blockDim.x) {
-        run_base[g] = run_rank[gptr[g]];
-        nruns[g] = run_rank[gptr[g + 1]] - run_base[g];
-    }
-}
-
-cudaError_t tp_run_bases(const long long *gptr, const long long *run_rank, int G, long long *run_base,
-                         long long *nruns, cudaStream_t s) {
-    run_bases_kernel<<<grid_for(G), 256, 0, s>>>(gptr, run_rank, G, run_base, nruns);
+cudaError_t tp_order_mark(const TpOrder &o, long long P, cudaStream_t s) {
+    tp_mark_kernel<<<grid_for(P), 256, 0, s>>>(o, P);
     note_launch();
     return cudaGetLastError();
 }
 
-int tp_merge_rounds(long long max_runs) {
-    int r = 0;
-    while ((1ll << r) < max_runs) ++r;
-    return r;
+cudaError_t tp_order_list(const TpOrder &o, long long P, long long n_subs, cudaStream_t s) {
+    tp_list_kernel<<<grid_for(P), 256, 0, s>>>(o, P);
+    tp_count_kernel<<<grid_for(n_subs), 256, 0, s>>>(o, P);
+    note_launch(2);
+    return cudaGetLastError();
 }
 
-// Thread t writes outputs [t*ITEMS, t*ITEMS + ITEMS) of round r: it finds
-// the graph and run of each output, the two run groups merged there, and the
-// merge-path split by binary search (A first on ties, so equal TPs stay
-// adjacent).  Graphs without TPs own no outputs.  cmp(a, b) orders two TPs
-// of one graph (here: their packed keys).
-template <typename Cmp>
-__global__ void tp_merge_graph_kernel(const long long *perm_in, long long *perm_out, const long long *bounds,
-                                      const long long *run_base, const long long *nruns, const long long *gptr,
-                                      int G, int r, long long P, Cmp cmp) {
-    const long long d0 = (blockIdx.x * (long long)blockDim.x + threadIdx.x) * TPM_ITEMS;
-    if (d0 >= P) return;
-    long long a_hi = 0, b_hi = -1, i = 0, j = 0;
-    for (int t = 0; t < TPM_ITEMS; ++t) {
-        const long long d = d0 + t;
-        if (d >= P) break;
-        if (d >= b_hi) {
-            const int gg = G > 1 ? (int)tp_slot(gptr, 0, G, d) : 0;
-            const long long rb = run_base[gg], nr = nruns[gg];
-            const long long q0 = tp_slot(bounds, rb, rb + nr - 1, d) - rb;
-            const long long m = q0 >> (r + 1);
-            const long long qa = m << (r + 1), qb = qa + (1ll << r), qe = (m + 1) << (r + 1);
-            const long long a_lo = bounds[rb + qa];
-            a_hi = bounds[rb + (qb < nr ? qb : nr)];
-            b_hi = bounds[rb + (qe < nr ? qe : nr)];
-            const long long na = a_hi - a_lo, nb = b_hi - a_hi, diag = d - a_lo;
-            long long lo = diag > nb ? diag - nb : 0, hi = diag < na ? diag : na;
-            while (lo < hi) {
-                const long long mid = (lo + hi) >> 1;
-                if (cmp(perm_in[a_lo + mid], perm_in[a_hi + diag - mid - 1]) <= 0) lo = mid + 1;
-                else hi = mid;
-            }
-            i = a_lo + lo;
-            j = a_hi + (diag - lo);
+cudaError_t tp_order_place(const TpOrder &o, long long P, long long n_subs, cudaStream_t s) {
+    tp_place_subs_kernel<<<grid_for(n_subs), 256, 0, s>>>(o, P);
+    tp_place_kernel<<<grid_for(P), 256, 0, s>>>(o, P);
+    note_launch(2);
+    return cudaGetLastError();
+}
+
+__global__ void __launch_bounds__(256) tp_plain_kernel(TpOrder o, long long P, const int *start, const long long *rank,
+                                                       int runs) {
+    long long *perm = o.perm[merge_rounds(runs) & 1];
+    for (long long i = blockIdx.x * 256ll + threadIdx.x; i < P; i += gridDim.x * 256ll) {
+        perm[i] = i;
+        o.pos_sub[i] = (int)(rank[i + 1] - 1);
+        if (start[i]) {
+            o.bounds[rank[i]] = i;
+            o.sub_info[rank[i]] = make_int4(0, runs, 0, 0);
         }
-        bool take_a;
-        if (i >= a_hi) take_a = false;
-        else if (j >= b_hi) take_a = true;
-        else take_a = cmp(perm_in[i], perm_in[j]) <= 0;
-        perm_out[d] = take_a ? perm_in[i++] : perm_in[j++];
+        if (i == 0) {
+            o.bounds[runs] = P;
+            *o.max_k = runs;
+        }
     }
 }
 
-struct KeyCmp {  // packed keys of one graph
-    const long long *koff;
-    const unsigned long long *key;
-    __device__ __forceinline__ int operator()(long long a, long long b) const {
-        return key_cmp_same_graph(a, b, koff, key);
-    }
-};
-
-cudaError_t tp_merge_graph_round_keys(const long long *perm_in, long long *perm_out, const long long *bounds,
-                                      const long long *run_base, const long long *nruns, const long long *gptr,
-                                      int G, int r, long long P, const long long *key_off,
-                                      const unsigned long long *key, cudaStream_t s) {
-    if (P <= 0) return cudaSuccess;
-    const long long threads = (P + TPM_ITEMS - 1) / TPM_ITEMS;
-    tp_merge_graph_kernel<<<(unsigned)((threads + 255) / 256), 256, 0, s>>>(perm_in, perm_out, bounds, run_base,
-                                                                           nruns, gptr, G, r, P,
-                                                                           KeyCmp{key_off, key});
+cudaError_t tp_order_plain(const TpOrder &o, long long P, const int *start, const long long *rank, long long runs,
+                           cudaStream_t s) {
+    tp_plain_kernel<<<grid_for(P), 256, 0, s>>>(o, P, start, rank, (int)runs);
     note_launch();
     return cudaGetLastError();
 }
 
-__global__ void key_len_kernel(const long long *tp_off, long long P, int vpw, long long *key_len) {
+constexpr int TPM_ITEMS = 4;  // outputs per thread of a merge round
+__global__ void __launch_bounds__(256) tp_merge_kernel(TpOrder o, int r, long long P) {
+    if (*o.max_k <= 1 << r) return;
+    const long long d0 = (blockIdx.x * 256ll + threadIdx.x) * TPM_ITEMS;
+    if (d0 < P) tp_merge_items<TPM_ITEMS>(o, r, P, d0);
+}
+
+cudaError_t tp_order_merge(const TpOrder &o, long long P, long long max_k, cudaStream_t s) {
+    if (P <= 0) return cudaSuccess;
+    const int rounds = merge_rounds(max_k);
+    for (int r = 0; r < rounds; ++r)
+        tp_merge_kernel<<<(unsigned)((P + 256ll * TPM_ITEMS - 1) / (256ll * TPM_ITEMS)), 256, 0, s>>>(o, r, P);
+    note_launch(rounds);
+    return cudaGetLastError();
+}
+
+__global__ void __launch_bounds__(256) tp_flags_kernel(TpOrder o, long long P, const long long *tp_off,
+                                                       long long *keep_len, int *keep) {
+    for (long long i = blockIdx.x * 256ll + threadIdx.x; i < P; i += gridDim.x * 256ll) {
+        const int k = tp_differs(o, i);
+        const long long x = o.perm[0][i];
+        keep[i] = k;
+        keep_len[i] = k ? tp_off[x + 1] - tp_off[x] : 0;
+    }
+}
+
+cudaError_t tp_order_flags(const TpOrder &o, long long P, const long long *tp_off, long long *keep_len, int *keep,
+                           cudaStream_t s) {
+    if (P <= 0) return cudaSuccess;
+    tp_flags_kernel<<<grid_for(P), 256, 0, s>>>(o, P, tp_off, keep_len, keep);
+    note_launch();
+    return cudaGetLastError();
+}
+
+template <int BLOCK>
+__global__ void __launch_bounds__(BLOCK) tree_slots_kernel(GraphDev g, int *arc_slot, int *end_slot) {
+    extern __shared__ int s_slots[];
+    tree_slots_block<BLOCK>(g, blockIdx.x, arc_slot, end_slot, s_slots);
+}
+
+cudaError_t tree_slots(const GraphDev &g, int *arc_slot, int *end_slot, cudaStream_t s) {
+    static_assert(3 * sizeof(int) * TPG_MAX_N <= 48 * 1024, "one graph's tables fit the default shared memory");
+    const size_t smem = 3 * sizeof(int) * (size_t)g.maxn;
+    if (g.maxn <= 256) tree_slots_kernel<128><<<g.G, 128, smem, s>>>(g, arc_slot, end_slot);
+    else tree_slots_kernel<1024><<<g.G, 1024, smem, s>>>(g, arc_slot, end_slot);
+    note_launch();
+    return cudaGetLastError();
+}
+
+__global__ void key_len_kernel(const long long *tp_off, long long P, int bits, long long *key_len) {
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < P;
          i += (long long)gridDim.x * blockDim.x)
-        key_len[i] = (tp_off[i + 1] - tp_off[i] + vpw - 1) / vpw;
+        key_len[i] = key_words(tp_off[i + 1] - tp_off[i], bits);
 }
 
 cudaError_t tp_key_lengths(const long long *tp_off, long long P, int bits, long long *key_len, cudaStream_t s) {
     if (P <= 0) return cudaSuccess;
-    key_len_kernel<<<grid_for(P), 256, 0, s>>>(tp_off, P, 64 / bits, key_len);
+    key_len_kernel<<<grid_for(P), 256, 0, s>>>(tp_off, P, bits, key_len);
     note_launch();
     return cudaGetLastError();
 }
@@ -303,26 +301,6 @@ cudaError_t tp_write_keys(const long long *tp_off, const int *tp_vert, long long
     long long blocks = (P + (256 / KEY_LANES) - 1) / (256 / KEY_LANES);
     if (blocks > (1 << 20)) blocks = 1 << 20;
     keys_kernel<<<(unsigned)blocks, 256, 0, s>>>(tp_off, tp_vert, P, bits, key_off, key);
-    note_launch();
-    return cudaGetLastError();
-}
-
-__global__ void dedup_keys_kernel(const long long *perm, long long P, const long long *tp_off, const long long *key_off,
-                                  const unsigned long long *key, const int *graph, long long *keep_len, int *keep) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < P;
-         i += (long long)gridDim.x * blockDim.x) {
-        const long long a = perm[i];
-        const int k = (i == 0) || key_cmp(perm[i - 1], a, key_off, key, graph) != 0;
-        keep[i] = k;
-        keep_len[i] = k ? tp_off[a + 1] - tp_off[a] : 0;
-    }
-}
-
-cudaError_t tp_dedup_flags_keys(const long long *perm, long long P, const long long *tp_off, const long long *key_off,
-                                const unsigned long long *key, const int *tp_graph, long long *keep_len, int *keep,
-                                cudaStream_t s) {
-    if (P <= 0) return cudaSuccess;
-    dedup_keys_kernel<<<grid_for(P), 256, 0, s>>>(perm, P, tp_off, key_off, key, tp_graph, keep_len, keep);
     note_launch();
     return cudaGetLastError();
 }

@@ -1,40 +1,37 @@
-// Per-graph TP run merging for the host-driven path (testpaths.cu).
+// TP ordering and keys of the host-driven path (testpaths.cu).
 #pragma once
 #include <cuda_runtime.h>
 
 #include "common.cuh"
+#include "tp_order_dev.cuh"
 
 namespace tpg {
 
-// run_base[g] / nruns[g]: the first run of graph g and its number of runs,
-// from the runs' exclusive prefix run_rank[P + 1] and the graph ranges
-// gptr[G + 1] of the (not yet merged) TP list.
-cudaError_t tp_run_bases(const long long *gptr, const long long *run_rank, int G, long long *run_base,
-                         long long *nruns, cudaStream_t s);
-// rounds that merge up to `max_runs` runs per graph
-int tp_merge_rounds(long long max_runs);
+// Order of the TPs (see tp_order_dev.cuh), in this sequence: mark, a scan of
+// o.start into o.sub_rank, list, count (slot_n zero before), a scan of slot_n
+// into slot_at, place; then the merge rounds and the flags, with the keys.
+// n_subs: an upper bound of the number of sub-runs.
+cudaError_t tp_order_mark(const TpOrder &o, long long P, cudaStream_t s);
+cudaError_t tp_order_list(const TpOrder &o, long long P, long long n_subs, cudaStream_t s);
+cudaError_t tp_order_place(const TpOrder &o, long long P, long long n_subs, cudaStream_t s);
+// one slot whose sub-runs start where `start` says (runs of them, `rank` its
+// exclusive prefix): bounds, sub_info, pos_sub, perm and max_k are set
+cudaError_t tp_order_plain(const TpOrder &o, long long P, const int *start, const long long *rank, long long runs,
+                           cudaStream_t s);
+// rounds 0 .. merge_rounds(max_k) - 1, max_k an upper bound
+cudaError_t tp_order_merge(const TpOrder &o, long long P, long long max_k, cudaStream_t s);
+// keep[i] = the TP at position i differs from the one before, its length if so
+cudaError_t tp_order_flags(const TpOrder &o, long long P, const long long *tp_off, long long *keep_len, int *keep,
+                           cudaStream_t s);
+// arc_slot[M], end_slot[G] of every graph (tree_slots_block)
+cudaError_t tree_slots(const GraphDev &g, int *arc_slot, int *end_slot, cudaStream_t s);
 
 // Packed comparison keys of the TPs (vertex v as v + 1 in `bits` = 8 or 16
-// bits, 64 / bits per word, most significant first; see key_cmp):
+// bits, 64 / bits per word, most significant first; see key_words):
 // key_len[i] = words of TP i, then (after a scan into key_off) the words.
 cudaError_t tp_key_lengths(const long long *tp_off, long long P, int bits, long long *key_len, cudaStream_t s);
 cudaError_t tp_write_keys(const long long *tp_off, const int *tp_vert, long long P, int bits, const long long *key_off,
                           unsigned long long *key, cudaStream_t s);
-// Round r of merging inside every graph: the graph's runs (its run q starts
-// at bounds[run_base[g] + q]; bounds[R] = P) are merged in groups, runs
-// [m 2^(r+1), m 2^(r+1) + 2^r) with the next 2^r, comparing packed keys;
-// after ceil(log2(runs)) rounds each graph is one sorted run.  Runs of
-// different graphs are never compared (the list is grouped by graph
-// already), so no graph ids are read.
-cudaError_t tp_merge_graph_round_keys(const long long *perm_in, long long *perm_out, const long long *bounds,
-                                      const long long *run_base, const long long *nruns, const long long *gptr,
-                                      int G, int r, long long P, const long long *key_off,
-                                      const unsigned long long *key, cudaStream_t s);
-// duplicate flags and kept lengths of the sorted TPs, on packed keys
-cudaError_t tp_dedup_flags_keys(const long long *perm, long long P, const long long *tp_off, const long long *key_off,
-                                const unsigned long long *key, const int *tp_graph, long long *keep_len, int *keep,
-                                cudaStream_t s);
-
 // packed keys (as tp_write_keys) of TP(p) for every PP p, read from the
 // TP's parts (prefix path, PP, suffix path) instead of a written TP list;
 // tp_off holds the TPs' offsets (for their lengths)

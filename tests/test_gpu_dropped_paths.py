@@ -49,6 +49,7 @@ def entered_everywhere(m):
 
 
 CASES = {
+    "n106": lambda: rings([50, 54]),  # (first: tables of 44 KB beside the kernel's own shared memory)
     "one-vertex-components": lambda: rings([1] * 12, tail=1),
     "rings": lambda: rings([3, 2, 4, 3], exits=2),
     "several-entries": lambda: rings([5, 6, 4], entries=3, exits=2, chords=[(0, 2), (3, 1)]),
