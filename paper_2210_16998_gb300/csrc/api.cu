@@ -1371,8 +1371,7 @@ int run_test_paths(tpg_cfg *g, Block **o_off, Block **o_vert, Block **o_gptr, lo
             cuda_err(tp_order_place(o, P, subs, s)) ||
             cuda_err(tp_key_lengths((const long long *)tp_off->p, P, kbits, g->s_len.as<long long>(), s)) ||
             cuda_err(scan_i64(g->s_len.as<long long>(), key_off, P, tmp, s)) ||
-            cuda_err(tp_write_keys_parts(pp_off, pp_vert, pp_graph, P, g->gd, (const long long *)tp_off->p, kbits,
-                                         key_off, key, s)) ||
+            cuda_err(tp_write_keys_parts(o, (const long long *)tp_off->p, key, P, s)) ||
             cuda_err(tp_order_merge(o, P, std::min<long long>(runs, g->maxn), s))) {
             rc = TPG_ECUDA;
             break;
@@ -1400,9 +1399,7 @@ int run_test_paths(tpg_cfg *g, Block **o_off, Block **o_vert, Block **o_gptr, lo
         if (!f_off || !f_vert || !f_gptr) { rc = TPG_ENOMEM; break; }
         if ((rc = ensure(g, g->s_i32[2], sizeof(int) * (T + 1)))) break;
         int *f_graph = g->s_i32[2].as<int>();
-        if (cuda_err(tp_assemble(perm, keep, keep_rank, P, pp_off, pp_vert, pp_graph, g->gd,
-                                 (const long long *)tp_off->p, keep_off, (long long *)f_off->p, (int *)f_vert->p, f_graph,
-                                 s))) {
+        if (cuda_err(tp_assemble(o, keep_off, keep_rank, (long long *)f_off->p, (int *)f_vert->p, f_graph, P, s))) {
             rc = TPG_ECUDA;
             break;
         }

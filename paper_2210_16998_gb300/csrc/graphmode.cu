@@ -197,50 +197,15 @@ __global__ void __launch_bounds__(GMB) gm_order_place(GmArgs a) {
     tp_place(a.order, gm_P_tp(a), blockIdx.x * (long long)GMB + threadIdx.x, gridDim.x * (long long)GMB);
 }
 
-// TP vertex at position p of TP i: prefix, PP, suffix
-struct TpParts {
-    const int *pre, *pp, *suf;
-    long long pl, plen;
-    __device__ __forceinline__ int at(long long p) const {
-        if (p < pl) return pre[p];
-        if (p < pl + plen) return pp[p - pl];
-        return suf[p - pl - plen];
-    }
-};
-
-constexpr int TP_LANES = 8;  // lanes per TP in the write and gather kernels
-
 // The packed comparison keys of every TP, read from its parts (the TPs
-// themselves are assembled once, in sorted order, by gm_tp_gather).
+// themselves are unpacked from them once, in sorted order, by gm_tp_gather).
+template <typename T>
 __global__ void __launch_bounds__(GMB) gm_tp_write(GmArgs a) {
     const long long P = gm_P_tp(a);
-    const GraphDev &g = a.g;
-    const int sub = threadIdx.x & (TP_LANES - 1);
-    const long long ngroups = (long long)gridDim.x * (GMB / TP_LANES);
-    const int bits = a.key_bits, vpw = 64 / bits;
-    for (long long i = blockIdx.x * (long long)(GMB / TP_LANES) + (threadIdx.x / TP_LANES); i < P; i += ngroups) {
-        const long long o0 = a.pp_off[i], o1 = a.pp_off[i + 1];
-        const int gid = g.G > 1 ? a.pp_graph[i] : 0;
-        const int vb = g.vgraph ? g.vbase[gid] : 0;
-        const int f = a.pp_vert[o0] + vb, l = a.pp_vert[o1 - 1] + vb;
-        TpParts t;
-        t.pl = g.pre_len[f] - 1;
-        t.plen = o1 - o0;
-        t.pre = g.pre_seq + g.pre_off[f];
-        t.pp = a.pp_vert + o0;
-        t.suf = g.suf_seq + g.suf_off[l] + 1;
-        const long long total = a.tp_off0[i + 1] - a.tp_off0[i];
-        const long long k0 = a.key_off[i], nw = a.key_off[i + 1] - k0;
-        for (long long w = sub; w < nw; w += TP_LANES) {
-            unsigned long long word = 0;
-            for (int q = 0; q < vpw; ++q) {
-                const long long p = w * vpw + q;
-                const unsigned long long v = p < total ? (unsigned long long)(t.at(p) + 1) : 0ull;
-                word = (word << bits) | v;
-            }
-            a.key[k0 + w] = word;
-        }
-    }
+    const int group = tp_group(P);
+    const long long step = gridDim.x * (GMB / 32ll) * group;
+    for (long long i0 = (blockIdx.x * (GMB / 32ll) + (threadIdx.x >> 5)) * group; i0 < P; i0 += step)
+        tp_write_keys_warp<T>(a.order, a.tp_off0, a.key, i0, group, P);
 }
 
 constexpr int GM_MERGE_ITEMS = 4;  // outputs per thread of a merge round
@@ -277,35 +242,15 @@ __device__ __forceinline__ long long gm_P_final(const GmArgs &a) {
     return gm_P_tp(a);
 }
 
-// The kept TPs in sorted order, each assembled from its parts (prefix path,
-// PP, suffix path) straight into its final place: the TP list is never
-// written in PP order.
+// The kept TPs in sorted order, each straight into its final place: the TP
+// list is never written in PP order.
+template <typename T>
 __global__ void __launch_bounds__(GMB) gm_tp_gather(GmArgs a) {
     const long long P = gm_P_final(a);
-    const long long *perm = a.order.perm[0];
-    const GraphDev &g = a.g;
-    const int sub = threadIdx.x & (TP_LANES - 1);
-    const long long ngroups = (long long)gridDim.x * (GMB / TP_LANES);
-    for (long long i = blockIdx.x * (long long)(GMB / TP_LANES) + (threadIdx.x / TP_LANES); i < P; i += ngroups) {
-        if (!a.keep[i]) continue;
-        const long long x = perm[i], rk = a.keep_rank[i];
-        const long long o0 = a.pp_off[x], o1 = a.pp_off[x + 1];
-        const int gid = g.G > 1 ? a.pp_graph[x] : 0;
-        const int vb = g.vgraph ? g.vbase[gid] : 0;
-        const int f = a.pp_vert[o0] + vb, l = a.pp_vert[o1 - 1] + vb;
-        TpParts t;
-        t.pl = g.pre_len[f] - 1;
-        t.plen = o1 - o0;
-        t.pre = g.pre_seq + g.pre_off[f];
-        t.pp = a.pp_vert + o0;
-        t.suf = g.suf_seq + g.suf_off[l] + 1;
-        const long long len = a.tp_off0[x + 1] - a.tp_off0[x], d0 = a.keep_off[i];
-        for (long long p = sub; p < len; p += TP_LANES) a.tp_vert[d0 + p] = t.at(p);
-        if (sub == 0) {
-            a.tp_graph[rk] = gid;
-            a.tp_off[rk] = d0;
-        }
-    }
+    const int group = tp_group(P);
+    const long long step = gridDim.x * (GMB / 32ll) * group;
+    for (long long i0 = (blockIdx.x * (GMB / 32ll) + (threadIdx.x >> 5)) * group; i0 < P; i0 += step)
+        tp_unpack_warp<T>(a.order, a.keep_off, a.keep_rank, a.tp_off, a.tp_vert, a.tp_graph, i0, group, P);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         const GmCounts *c = a.counts;
         a.tp_off[P ? c->T : 0] = P ? c->TV : 0;
@@ -378,7 +323,8 @@ cudaError_t gm_enqueue_tp(const GmArgs &a, cudaStream_t s) {
     if ((e = scan_i64(a.order.slot_n, a.order.slot_at, a.slots, a.scan_tmp, s))) return e;
     gm_order_place_subs<<<grid, GMB, 0, s>>>(a);
     gm_order_place<<<grid, GMB, 0, s>>>(a);
-    gm_tp_write<<<grid, GMB, 0, s>>>(a);
+    if (a.key_bits == 8) gm_tp_write<unsigned char><<<grid, GMB, 0, s>>>(a);
+    else gm_tp_write<unsigned short><<<grid, GMB, 0, s>>>(a);
     note_launch(3);
     for (int r = 0; r < a.tp_rounds; ++r) gm_tp_merge_round<<<grid, GMB, 0, s>>>(a, r);
     gm_tp_dedup<<<grid, GMB, 0, s>>>(a);
@@ -388,7 +334,8 @@ cudaError_t gm_enqueue_tp(const GmArgs &a, cudaStream_t s) {
     if ((e = gm_scan<int>(a.keep, a.keep_rank, &a.counts->P, a.P_cap, a.scan_tmp, nullptr, a.num_sms, s)))
         return e;
     gm_tp_totals<<<1, 32, 0, s>>>(a);
-    gm_tp_gather<<<grid, GMB, 0, s>>>(a);
+    if (a.key_bits == 8) gm_tp_gather<unsigned char><<<grid, GMB, 0, s>>>(a);
+    else gm_tp_gather<unsigned short><<<grid, GMB, 0, s>>>(a);
     gm_graph_ptr<<<grid, GMB, 0, s>>>(a.tp_graph, &a.counts->T, a.P_cap, a.g.G, a.tp_gptr, a.counts,
                                       GM_ENUM_FAILED | GM_OVF_PP | GM_OVF_PPV | GM_UNREACH | GM_OVF_TPV0 | GM_OVF_TPV);
     note_launch(3);

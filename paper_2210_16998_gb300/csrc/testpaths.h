@@ -34,15 +34,13 @@ cudaError_t tp_write_keys(const long long *tp_off, const int *tp_vert, long long
                           unsigned long long *key, cudaStream_t s);
 // packed keys (as tp_write_keys) of TP(p) for every PP p, read from the
 // TP's parts (prefix path, PP, suffix path) instead of a written TP list;
-// tp_off holds the TPs' offsets (for their lengths)
-cudaError_t tp_write_keys_parts(const long long *pp_off, const int *pp_vert, const int *pp_graph, long long P,
-                                const GraphDev &g, const long long *tp_off, int bits, const long long *key_off,
-                                unsigned long long *key, cudaStream_t s);
-// as tp_gather, but every kept TP is assembled from its parts
-cudaError_t tp_assemble(const long long *perm, const int *keep, const long long *keep_rank, long long P,
-                        const long long *pp_off, const int *pp_vert, const int *pp_graph, const GraphDev &g,
-                        const long long *tp_off, const long long *keep_off, long long *final_off, int *out_vert,
-                        int *out_graph, cudaStream_t s);
+// tp_off holds the TPs' offsets (for their lengths), o.key_off the keys'
+cudaError_t tp_write_keys_parts(const TpOrder &o, const long long *tp_off, unsigned long long *key, long long P,
+                                cudaStream_t s);
+// the kept TPs in sorted order (o.perm[0], lengths between keep_off[P + 1]),
+// unpacked from their keys into their final places
+cudaError_t tp_assemble(const TpOrder &o, const long long *keep_off, const long long *keep_rank, long long *final_off,
+                        int *out_vert, int *out_graph, long long P, cudaStream_t s);
 // map[perm[i]] = the final index of sorted TP i (keep_rank[i] if it is kept,
 // else that of the kept TP it duplicates, keep_rank[i] - 1); with perm null
 // the identity map[i] = i

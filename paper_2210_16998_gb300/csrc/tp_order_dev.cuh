@@ -288,4 +288,88 @@ __device__ __forceinline__ bool tp_differs(const TpOrder &o, long long i) {
                          o.bits) != 0;
 }
 
+// TPs that a warp of the two kernels below takes at a time, of P: their parts
+// are gathered by a lane each, then half a warp goes along one TP.
+constexpr int TP_WARPS = 9728;  // 64 warps on each of 152 SMs
+__host__ __device__ inline int tp_group(long long P) {
+    const long long per = (P + TP_WARPS - 1) / TP_WARPS;
+    return per < 2 ? 2 : per > 32 ? 32 : (int)((per + 1) & ~1ll);
+}
+
+// Packed keys of the TPs [i0, i0 + group) cut off at P, by one warp: each
+// vertex is read once from its part (prefix path, PP, suffix path) and stored
+// at its place in its word (words hold the first vertex in their high bits).
+template <typename T>
+__device__ __forceinline__ void tp_write_keys_warp(const TpOrder &o, const long long *tp_off, unsigned long long *key,
+                                                   long long i0, int group, long long P) {
+    constexpr int VPW = 8 / sizeof(T);
+    const GraphDev &g = o.g;
+    const int lane = threadIdx.x & 31, sub = lane & 15;
+    const long long i = i0 + lane;
+    // lane l's TP: where a position p of it lies, per part, and its key
+    const int *pre = nullptr, *pp = nullptr, *suf = nullptr;
+    int pl = 0, pe = 0, len = 0;
+    long long k0 = 0;
+    if (lane < group && i < P) {
+        const long long o0 = o.pp_off[i], o1 = o.pp_off[i + 1];
+        const int vb = g.vgraph ? g.vbase[o.pp_graph ? o.pp_graph[i] : 0] : 0;
+        const int f = o.pp_vert[o0] + vb, l = o.pp_vert[o1 - 1] + vb;
+        len = (int)(tp_off[i + 1] - tp_off[i]);
+        k0 = o.key_off[i];
+        pl = g.pre_len[f] - 1;
+        pe = pl + (int)(o1 - o0);
+        pre = g.pre_seq + g.pre_off[f];
+        pp = o.pp_vert + o0 - pl;
+        suf = g.suf_seq + g.suf_off[l] + 1 - pe;
+    }
+    for (int t = 0; t < group; t += 2) {
+        const int src = t + (lane >> 4);
+        const int *tpre = (const int *)__shfl_sync(0xffffffffu, (unsigned long long)pre, src);
+        const int *tpp = (const int *)__shfl_sync(0xffffffffu, (unsigned long long)pp, src);
+        const int *tsuf = (const int *)__shfl_sync(0xffffffffu, (unsigned long long)suf, src);
+        const int tpl = __shfl_sync(0xffffffffu, pl, src), tpe = __shfl_sync(0xffffffffu, pe, src);
+        const int tlen = __shfl_sync(0xffffffffu, len, src);
+        T *dst = (T *)(key + __shfl_sync(0xffffffffu, k0, src));
+        const int end = tlen > 0 ? (tlen / VPW + 1) * VPW : 0;
+#pragma unroll 4
+        for (int p = sub; p < end; p += 16) {
+            int v = 0;
+            if (p < tlen) v = (p < tpl ? tpre : p < tpe ? tpp : tsuf)[p] + 1;
+            dst[p ^ (VPW - 1)] = (T)v;
+        }
+    }
+}
+
+// The kept TPs of the sorted positions [i0, i0 + group), unpacked from their
+// keys straight into their final places (contiguous ones), by one warp.
+template <typename T>
+__device__ __forceinline__ void tp_unpack_warp(const TpOrder &o, const long long *keep_off, const long long *keep_rank,
+                                               long long *final_off, int *out_vert, int *out_graph, long long i0,
+                                               int group, long long P) {
+    constexpr int VPW = 8 / sizeof(T);
+    const int lane = threadIdx.x & 31, sub = lane & 15;
+    const long long i = i0 + lane;
+    const T *from = nullptr;
+    long long d0 = 0;
+    int len = 0;
+    if (lane < group && i < P) {
+        d0 = keep_off[i];
+        len = (int)(keep_off[i + 1] - d0);  // 0: a duplicate
+        if (len > 0) {
+            const long long x = o.perm[0][i], r = keep_rank[i];
+            from = (const T *)(o.key + o.key_off[x]);
+            out_graph[r] = o.pp_graph ? o.pp_graph[x] : 0;
+            final_off[r] = d0;
+        }
+    }
+    for (int t = 0; t < group; t += 2) {
+        const int src = t + (lane >> 4);
+        const T *tfrom = (const T *)__shfl_sync(0xffffffffu, (unsigned long long)from, src);
+        const int tlen = __shfl_sync(0xffffffffu, len, src);
+        int *dst = out_vert + __shfl_sync(0xffffffffu, d0, src);
+#pragma unroll 4
+        for (int p = sub; p < tlen; p += 16) dst[p] = (int)tfrom[p ^ (VPW - 1)] - 1;
+    }
+}
+
 }  // namespace tpg
