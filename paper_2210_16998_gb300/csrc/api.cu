@@ -402,6 +402,7 @@ struct tpg_cfg {
     DevBuf pre_len, suf_len, pre_off, suf_off, pre_seq, suf_seq;
     DevBuf smask, pmask;  // successor / predecessor bitsets (bitsets of <= MASK_MAX_W words)
     DevBuf arc_slot, end_slot;  // where a TP can leave the entry's BFS tree (tree_slots_block)
+    DevBuf thin;                // counts of the walks of thin graphs
     DevBuf tp_subs, tp_slots;   // the TP ordering's tables
     DevBuf cmask, dflags, xinfo, dropD, dropX, drop_lvl;  // paths that cannot become PPs (DoomDev), same graphs
     GraphDev gd{};
@@ -445,6 +446,7 @@ struct tpg_cfg {
     } gp;
     long long out_cap[4] = {0, 0, 0, 0};  // explicit output capacities P, V, TV0, TV (0 = last run)
     unsigned long long *root_counts = nullptr;  // set while a counting run is in progress
+    bool frontier_only = false;  // capacities, a tile shape, a split or a wait limit were set: they are the frontier's
     bool trace_on = false;  // record a per-level trace of the frontier launches
     DevBuf trace;
     std::vector<long long> h_trace;  // the last call's trace, LEVEL_TRACE_WORDS per level
@@ -533,7 +535,7 @@ void destroy_cfg(tpg_cfg *g) {
     }
     DevBuf *all[] = {&g->rp, &g->col, &g->prp, &g->pcol, &g->vgraph, &g->vbase, &g->entry, &g->exitv,
                      &g->tbl_base, &g->dist, &g->pred, &g->pre_len, &g->suf_len, &g->pre_off, &g->suf_off,
-                     &g->smask, &g->pmask, &g->arc_slot, &g->end_slot, &g->tp_subs, &g->tp_slots, &g->cmask, &g->dflags, &g->xinfo, &g->dropD, &g->dropX, &g->drop_lvl,
+                     &g->smask, &g->pmask, &g->arc_slot, &g->end_slot, &g->thin, &g->tp_subs, &g->tp_slots, &g->cmask, &g->dflags, &g->xinfo, &g->dropD, &g->dropX, &g->drop_lvl,
                      &g->pre_seq, &g->suf_seq, &g->tfl[0], &g->tfl[1], &g->tvis[0], &g->tvis[1], &g->tcnt[0], &g->tcnt[1],
                      &g->levels, &g->agg, &g->ctl, &g->s_keys[0], &g->s_keys[1],
                      &g->s_refs[0], &g->s_refs[1], &g->s_len, &g->s_tmp, &g->s_i32[0], &g->s_i32[1],
@@ -1006,9 +1008,135 @@ private:
     bool running_ = false;
 };
 
+// Walks are tried above this many vertices: below, a level's bitsets fit the
+// frontier's registers, and it has at most as many levels.
+constexpr int THIN_MIN_N = 256;
+
+// Blocks of P PPs with V vertices, kept by the handle.
+int alloc_pps(tpg_cfg *g, long long P, long long V) {
+    cudaStream_t s = g->stream;
+    Block *off = block_new(g->fns, sizeof(long long) * (P + 1), s);
+    Block *vert = block_new(g->fns, sizeof(int) * std::max<long long>(V, 1), s);
+    Block *gptr = block_new(g->fns, sizeof(long long) * (g->G + 1), s);
+    Block *pgraph = g->G > 1 ? block_new(g->fns, sizeof(int) * std::max<long long>(P, 1), s) : nullptr;
+    if (!off || !vert || !gptr || (g->G > 1 && !pgraph)) {
+        block_unref(off);
+        block_unref(vert);
+        block_unref(gptr);
+        block_unref(pgraph);
+        return TPG_ENOMEM;
+    }
+    g->pp_off = off;
+    g->pp_vert = vert;
+    g->pp_gptr = gptr;
+    g->pp_graph = pgraph;
+    return ensure(g, g->pp_ends, sizeof(int2) * std::max<long long>(P, 1));
+}
+
+// The graphs' ranges of the PP list.
+int pp_graph_ranges(tpg_cfg *g, long long P) {
+    if (g->G > 1) {
+        CK(graph_ptr_from_ids((const int *)g->pp_graph->p, P, g->G, (long long *)g->pp_gptr->p, g->stream));
+    } else {
+        long long *h = (long long *)g->h_small;
+        h[0] = 0;
+        h[1] = P;
+        CK(cudaMemcpyAsync(g->pp_gptr->p, h, 2 * sizeof(long long), cudaMemcpyHostToDevice, g->stream));
+    }
+    return TPG_OK;
+}
+
+// The PPs of graphs above 256 vertices by walks (thin.cu), unless their paths
+// multiply: *done tells.
+int run_thin(tpg_cfg *g, bool *done) {
+    cudaStream_t s = g->stream;
+    *done = false;
+    const size_t L = (size_t)g->max_levels, N = (size_t)g->N;
+    const size_t head = sizeof(long long) * (1 + 2 * L);
+    RC(ensure(g, g->thin, head + sizeof(long long) * 4 * (N + 1)));
+    RC(ensure(g, g->s_tmp, sizeof(long long) * scan_tmp_elems(N + 1)));
+    long long *stage = (long long *)level_stage(g, head);
+    if (!stage) {  // no page-locked memory: an ordinary buffer
+        g->h_lvl_plain.resize(head);
+        stage = (long long *)g->h_lvl_plain.data();
+    }
+    ThinArgs a{};
+    a.g = g->gd;
+    long long *p = g->thin.as<long long>();
+    a.stop = (int *)p;
+    a.paths = p + 1;
+    a.pps = a.paths + L;
+    a.root_pp = a.pps + L;
+    a.root_ppv = a.root_pp + N + 1;
+    long long *pp_at = a.root_ppv + N + 1, *ppv_at = pp_at + N + 1;
+    a.pp_at = pp_at;
+    a.ppv_at = ppv_at;
+    CK(cudaEventRecord(g->ev[0], s));
+    CK(cudaMemsetAsync(p, 0, head, s));
+    CK(thin_count(a, s));
+    CK(cudaEventRecord(g->ev[1], s));
+    CK(cudaMemcpyAsync(stage, p, head, cudaMemcpyDeviceToHost, s));
+    CK(cudaStreamSynchronize(s));
+    if (*(const int *)stage) return TPG_OK;
+    float ms = 0.f;
+    cudaEventElapsedTime(&ms, g->ev[0], g->ev[1]);
+    long long P = 0, V = 0, nodes = 0, peak = 0, paths = 0;
+    int K = 0, pp_levels = 0;
+    for (int k = 1; k < g->max_levels; ++k) {
+        const long long pps = stage[1 + L + k];
+        paths += stage[1 + k];
+        nodes += paths;
+        peak = std::max(peak, paths);
+        if (paths > 0) K = k;
+        pp_levels += pps > 0;
+        P += pps;
+        V += k * pps;
+    }
+    g->last_nodes = nodes;
+    g->last_peak = peak;
+    g->stats.t_enumerate_ms = ms;
+    g->stats.attempts = 1;
+    g->stats.enumerate_grid = g->N;
+    g->stats.tile_block = 32;
+    g->stats.tile_items = 1;
+    g->stats.simple_paths = nodes;
+    g->stats.levels = K;
+    g->stats.peak_level_nodes = peak;
+    g->stats.pp_levels = pp_levels;
+    g->stats.prime_paths = P;
+    g->stats.pp_vertices = V;
+    g->stats.bitset_words = g->W;
+    g->stats.arena_bytes_used = g->stats.arena_bytes_alloc = 0;  // (no path is stored)
+    g->stats.frontier_bytes_alloc = 0;
+    RC(alloc_pps(g, P, V));
+    a.off = (long long *)g->pp_off->p;
+    a.vert = (int *)g->pp_vert->p;
+    a.pgraph = g->pp_graph ? (int *)g->pp_graph->p : nullptr;
+    a.ends = g->pp_ends.as<int2>();
+    long long *tmp = g->s_tmp.as<long long>();
+    CK(cudaEventRecord(g->ev[2], s));
+    CK(scan_i64(a.root_pp, pp_at, g->N, tmp, s));
+    CK(scan_i64(a.root_ppv, ppv_at, g->N, tmp, s));
+    CK(thin_write(a, s));
+    RC(pp_graph_ranges(g, P));
+    CK(cudaEventRecord(g->ev[3], s));
+    CK(cudaStreamSynchronize(s));
+    cudaEventElapsedTime(&g->stats.t_order_ms, g->ev[2], g->ev[3]);
+    g->P = P;
+    g->V = V;
+    g->pp_valid = true;
+    *done = true;
+    return TPG_OK;
+}
+
 int run_prime_paths(tpg_cfg *g) {
     cudaStream_t s = g->stream;
     drop_cache(g);
+    if (g->maxn > THIN_MIN_N && !g->frontier_only && !g->trace_on) {
+        bool done = false;
+        RC(run_thin(g, &done));
+        if (done) return TPG_OK;
+    }
     RC(enumerate_levels(g));
     DropCount drops(g);
     CK(drops.start());
@@ -1040,23 +1168,9 @@ int run_prime_paths(tpg_cfg *g) {
     g->stats.arena_bytes_alloc = seg_bytes;
     g->stats.frontier_bytes_alloc = 2 * g->lvl_cap * (long long)(sizeof(int2) + 4 * g->W);
 
-    Block *off = block_new(g->fns, sizeof(long long) * (P + 1), s);
-    Block *vert = block_new(g->fns, sizeof(int) * std::max<long long>(V, 1), s);
-    Block *gptr = block_new(g->fns, sizeof(long long) * (g->G + 1), s);
-    Block *pgraph = g->G > 1 ? block_new(g->fns, sizeof(int) * std::max<long long>(P, 1), s) : nullptr;
-    if (!off || !vert || !gptr || (g->G > 1 && !pgraph)) {
-        block_unref(off);
-        block_unref(vert);
-        block_unref(gptr);
-        block_unref(pgraph);
-        return TPG_ENOMEM;
-    }
-    g->pp_off = off;
-    g->pp_vert = vert;
-    g->pp_gptr = gptr;
-    g->pp_graph = pgraph;
+    RC(alloc_pps(g, P, V));
+    Block *off = g->pp_off, *vert = g->pp_vert, *pgraph = g->pp_graph;
     const LevelRec *dlev = g->levels.as<LevelRec>();
-    RC(ensure(g, g->pp_ends, sizeof(int2) * std::max<long long>(P, 1)));
     int2 *ends = g->pp_ends.as<int2>();
     CK(cudaEventRecord(g->ev[2], s));
     if (P == 0) {
@@ -1081,14 +1195,7 @@ int run_prime_paths(tpg_cfg *g) {
         CK(pp_materialize(refs, nullptr, 0, P, (const long long *)off->p, dlev, g->max_levels, g->gd, (int *)vert->p,
                           pgraph ? (int *)pgraph->p : nullptr, s, ends));
     }
-    if (g->G > 1) {
-        CK(graph_ptr_from_ids(pgraph ? (const int *)pgraph->p : nullptr, P, g->G, (long long *)gptr->p, s));
-    } else {
-        long long *h = (long long *)g->h_small;
-        h[0] = 0;
-        h[1] = P;
-        CK(cudaMemcpyAsync(gptr->p, h, 2 * sizeof(long long), cudaMemcpyHostToDevice, s));
-    }
+    RC(pp_graph_ranges(g, P));
     CK(cudaEventRecord(g->ev[3], s));
     CK(drops.fetch());
     CK(cudaStreamSynchronize(s));
@@ -3046,6 +3153,7 @@ int tpg_set_tile_shape(tpg_cfg *g, int32_t block, int32_t items) {
     const EnumShape sh{block, items};
     if (!enum_shape_supported(g->W, sh)) return TPG_EINVAL;
     g->shape = sh;
+    g->frontier_only = true;
     return TPG_OK;
 }
 
@@ -3053,12 +3161,14 @@ int tpg_set_work_split(tpg_cfg *g, int32_t split) {
     if (!is_cfg(g)) return TPG_EHANDLE;
     if (split < 1 || split > 4) return TPG_EINVAL;
     g->split = split;
+    g->frontier_only = true;
     return TPG_OK;
 }
 
 int tpg_set_wait_limit(tpg_cfg *g, int64_t ns) {
     if (!is_cfg(g)) return TPG_EHANDLE;
     g->spin_ns = ns < 0 ? SPIN_LIMIT_NS : (unsigned long long)ns;
+    if (ns >= 0) g->frontier_only = true;
     return TPG_OK;
 }
 
@@ -3068,6 +3178,7 @@ int tpg_set_capacity(tpg_cfg *g, int64_t nodes, int64_t level_nodes, int64_t pri
     g->node_cap = nodes;
     g->lvl_cap = level_nodes;
     g->pp_cap = prime_paths;
+    g->frontier_only = true;
     return TPG_OK;
 }
 

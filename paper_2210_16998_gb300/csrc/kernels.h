@@ -134,6 +134,24 @@ cudaError_t enum_reset(const GraphDev &g, const DoomDev &dm, long long tbl, Leve
 cudaError_t doom_count(const GraphDev &g, const DoomDev &dm, const LevelRec *levels, int max_levels,
                        unsigned long long *level, cudaStream_t s);
 
+// thin.cu
+// Walks of thin graphs.  thin_count: paths (as differences: their running sums)
+// and PPs by number of vertices (zero before), PPs and their vertices by first vertex, or *stop (zero before) is set
+// and nothing else is of use; thin_write: the PPs, from the prefixes of the
+// latter two.
+struct ThinArgs {
+    GraphDev g;
+    int *stop;
+    long long *paths, *pps;              // [max_levels]
+    long long *root_pp, *root_ppv;       // [N]
+    const long long *pp_at, *ppv_at;     // [N + 1] their prefixes
+    long long *off;                      // [PPs + 1]
+    int *vert, *pgraph;                  // pgraph may be null
+    int2 *ends;                          // (first, last) local vertex of each PP
+};
+cudaError_t thin_count(const ThinArgs &a, cudaStream_t s);
+cudaError_t thin_write(const ThinArgs &a, cudaStream_t s);
+
 // order.cu
 // canonical ordering of PP references across levels (ancestor-index merge)
 cudaError_t order_init_run(const int *pp_refs_level, int level, long long n, int *keys,
