@@ -1466,7 +1466,7 @@ int run_test_paths(tpg_cfg *g, Block **o_off, Block **o_vert, Block **o_gptr, lo
         const int kbits = g->maxn <= 255 ? 8 : 16;
         const long long K_ub = TV / (64 / kbits) + P + 1;
         if ((rc = tp_order_arrays(g, g->tp_subs, g->tp_slots, subs, &o)) ||
-            (rc = ensure(g, g->tp_key, sizeof(unsigned long long) * K_ub)))
+            (rc = ensure(g, g->tp_key, sizeof(unsigned long long) * (K_ub + KEY_PAD))))
             break;
         long long *key_off = g->tp_key_off.as<long long>();
         unsigned long long *key = g->tp_key.as<unsigned long long>();
@@ -1590,7 +1590,7 @@ int capture_plan(tpg_cfg *g) {
     const int key_bits = g->maxn <= 255 ? 8 : 16;
     const long long K_cap = p.TV0_cap / (64 / key_bits) + Pc + 1;
     RC(ensure(g, p.key_off, sizeof(long long) * (Pc + 1)));
-    RC(ensure(g, p.key, sizeof(unsigned long long) * K_cap));
+    RC(ensure(g, p.key, sizeof(unsigned long long) * (K_cap + KEY_PAD)));
     RC(alloc_fixed_workspace(g));
     p.pp_off = block_new(g->fns, sizeof(long long) * (Pc + 1), s);
     p.pp_vert = block_new(g->fns, sizeof(int) * p.V_cap, s);
@@ -2420,7 +2420,7 @@ static int sort_paths(tpg_cfg *g, const long long *off, const int *vert, long lo
     long long T = 0, TV = 0;
     do {
         if ((rc = ensure(g, klen, sizeof(long long) * (n + 1))) || (rc = ensure(g, koff, sizeof(long long) * (n + 1))) ||
-            (rc = ensure(g, key, sizeof(unsigned long long) * K_ub)) || (rc = ensure(g, rrank, sizeof(long long) * (n + 1))) ||
+            (rc = ensure(g, key, sizeof(unsigned long long) * (K_ub + KEY_PAD))) || (rc = ensure(g, rrank, sizeof(long long) * (n + 1))) ||
             (rc = ensure(g, pos, sizeof(int) * n)) ||
             (rc = ensure(g, perm0, sizeof(long long) * n)) || (rc = ensure(g, perm1, sizeof(long long) * n)) ||
             (rc = ensure(g, keep, sizeof(int) * n)) || (rc = ensure(g, keep_len, sizeof(long long) * n)) ||

@@ -209,19 +209,21 @@ __global__ void __launch_bounds__(GMB) gm_tp_write(GmArgs a) {
 }
 
 constexpr int GM_MERGE_ITEMS = 4;  // outputs per thread of a merge round
+template <int BITS>
 __global__ void __launch_bounds__(GMB) gm_tp_merge_round(GmArgs a, int r) {
     const long long P = gm_P_tp(a);
     if (P <= 0 || *a.order.max_k <= 1 << r) return;
     const long long step = (long long)gridDim.x * GMB * GM_MERGE_ITEMS;
     for (long long d0 = (blockIdx.x * (long long)GMB + threadIdx.x) * GM_MERGE_ITEMS; d0 < P; d0 += step)
-        tp_merge_items<GM_MERGE_ITEMS>(a.order, r, P, d0);
+        tp_merge_items<GM_MERGE_ITEMS, BITS>(a.order, r, P, d0);
 }
 
+template <int BITS>
 __global__ void __launch_bounds__(GMB) gm_tp_dedup(GmArgs a) {
     const long long P = gm_P_tp(a);
     for (long long i = blockIdx.x * (long long)GMB + threadIdx.x; i < P; i += (long long)gridDim.x * GMB) {
         const long long x = a.order.perm[0][i];
-        const int k = tp_differs(a.order, i);
+        const int k = tp_differs<BITS>(a.order, i);
         a.keep[i] = k;
         a.tp_len[i] = k ? a.tp_off0[x + 1] - a.tp_off0[x] : 0;
     }
@@ -326,8 +328,12 @@ cudaError_t gm_enqueue_tp(const GmArgs &a, cudaStream_t s) {
     if (a.key_bits == 8) gm_tp_write<unsigned char><<<grid, GMB, 0, s>>>(a);
     else gm_tp_write<unsigned short><<<grid, GMB, 0, s>>>(a);
     note_launch(3);
-    for (int r = 0; r < a.tp_rounds; ++r) gm_tp_merge_round<<<grid, GMB, 0, s>>>(a, r);
-    gm_tp_dedup<<<grid, GMB, 0, s>>>(a);
+    for (int r = 0; r < a.tp_rounds; ++r) {
+        if (a.key_bits == 8) gm_tp_merge_round<8><<<grid, GMB, 0, s>>>(a, r);
+        else gm_tp_merge_round<16><<<grid, GMB, 0, s>>>(a, r);
+    }
+    if (a.key_bits == 8) gm_tp_dedup<8><<<grid, GMB, 0, s>>>(a);
+    else gm_tp_dedup<16><<<grid, GMB, 0, s>>>(a);
     note_launch(a.tp_rounds + 1);
     if ((e = gm_scan<long long>(a.tp_len, a.keep_off, &a.counts->P, a.P_cap, a.scan_tmp, nullptr, a.num_sms, s)))
         return e;

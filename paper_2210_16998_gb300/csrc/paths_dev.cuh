@@ -11,15 +11,35 @@ namespace tpg {
 // Comparing word by word orders the sequences lexicographically with a proper
 // prefix first, and equal keys mean equal sequences.
 __host__ __device__ inline long long key_words(long long len, int bits) { return len / (64 / bits) + 1; }
-__device__ __forceinline__ bool key_end(unsigned long long word, int bits) {
-    return (word & ((1ull << bits) - 1)) == 0ull;
+template <int BITS>
+__device__ __forceinline__ bool key_end(unsigned long long word) {
+    return (word & ((1ull << BITS) - 1)) == 0ull;
 }
 
-__device__ __forceinline__ int key_cmp_words(const unsigned long long *a, const unsigned long long *b, int bits) {
-    for (;; ++a, ++b) {
+// Long common parts of wide keys (up to 1024 words) are read four words a round
+// trip, so up to KEY_PAD words past the end of the shorter key; keys of 8 bits
+// have at most 64 words, a few of which are read (1100-vertex chain: merging
+// 1.26 -> 0.51 ms).
+constexpr int KEY_PAD = 4;
+template <int BITS>
+__device__ __forceinline__ int key_cmp_words(const unsigned long long *a, const unsigned long long *b) {
+    for (int i = 0; BITS == 8 || i < 2; ++i, ++a, ++b) {
         const unsigned long long x = *a, y = *b;
         if (x != y) return x < y ? -1 : 1;
-        if (key_end(x, bits)) return 0;
+        if (key_end<BITS>(x)) return 0;
+    }
+    for (;; a += 4, b += 4) {
+        unsigned long long x[4], y[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            x[i] = a[i];
+            y[i] = b[i];
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            if (x[i] != y[i]) return x[i] < y[i] ? -1 : 1;
+            if (key_end<BITS>(x[i])) return 0;
+        }
     }
 }
 

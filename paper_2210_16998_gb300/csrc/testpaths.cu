@@ -213,25 +213,30 @@ cudaError_t tp_order_plain(const TpOrder &o, long long P, const int *start, cons
 }
 
 constexpr int TPM_ITEMS = 4;  // outputs per thread of a merge round
+template <int BITS>
 __global__ void __launch_bounds__(256) tp_merge_kernel(TpOrder o, int r, long long P) {
     if (*o.max_k <= 1 << r) return;
     const long long d0 = (blockIdx.x * 256ll + threadIdx.x) * TPM_ITEMS;
-    if (d0 < P) tp_merge_items<TPM_ITEMS>(o, r, P, d0);
+    if (d0 < P) tp_merge_items<TPM_ITEMS, BITS>(o, r, P, d0);
 }
 
 cudaError_t tp_order_merge(const TpOrder &o, long long P, long long max_k, cudaStream_t s) {
     if (P <= 0) return cudaSuccess;
     const int rounds = merge_rounds(max_k);
-    for (int r = 0; r < rounds; ++r)
-        tp_merge_kernel<<<(unsigned)((P + 256ll * TPM_ITEMS - 1) / (256ll * TPM_ITEMS)), 256, 0, s>>>(o, r, P);
+    const unsigned grid = (unsigned)((P + 256ll * TPM_ITEMS - 1) / (256ll * TPM_ITEMS));
+    for (int r = 0; r < rounds; ++r) {
+        if (o.bits == 8) tp_merge_kernel<8><<<grid, 256, 0, s>>>(o, r, P);
+        else tp_merge_kernel<16><<<grid, 256, 0, s>>>(o, r, P);
+    }
     note_launch(rounds);
     return cudaGetLastError();
 }
 
+template <int BITS>
 __global__ void __launch_bounds__(256) tp_flags_kernel(TpOrder o, long long P, const long long *tp_off,
                                                        long long *keep_len, int *keep) {
     for (long long i = blockIdx.x * 256ll + threadIdx.x; i < P; i += gridDim.x * 256ll) {
-        const int k = tp_differs(o, i);
+        const int k = tp_differs<BITS>(o, i);
         const long long x = o.perm[0][i];
         keep[i] = k;
         keep_len[i] = k ? tp_off[x + 1] - tp_off[x] : 0;
@@ -241,7 +246,8 @@ __global__ void __launch_bounds__(256) tp_flags_kernel(TpOrder o, long long P, c
 cudaError_t tp_order_flags(const TpOrder &o, long long P, const long long *tp_off, long long *keep_len, int *keep,
                            cudaStream_t s) {
     if (P <= 0) return cudaSuccess;
-    tp_flags_kernel<<<grid_for(P), 256, 0, s>>>(o, P, tp_off, keep_len, keep);
+    if (o.bits == 8) tp_flags_kernel<8><<<grid_for(P), 256, 0, s>>>(o, P, tp_off, keep_len, keep);
+    else tp_flags_kernel<16><<<grid_for(P), 256, 0, s>>>(o, P, tp_off, keep_len, keep);
     note_launch();
     return cudaGetLastError();
 }

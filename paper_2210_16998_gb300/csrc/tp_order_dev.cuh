@@ -209,7 +209,7 @@ __device__ __forceinline__ void tp_place(const TpOrder &o, long long P, long lon
 // sub-runs, sub-runs [m 2^(r+1), m 2^(r+1) + 2^r) with the next 2^r.  The split
 // is found by binary search, then the heads' first unshared words stay in
 // registers (A first on ties, so equal TPs stay adjacent).
-template <int ITEMS>
+template <int ITEMS, int BITS>
 __device__ __forceinline__ void tp_merge_items(const TpOrder &o, int r, long long P, long long d0) {
     const long long *in = nullptr;
     long long *out = nullptr;
@@ -252,8 +252,8 @@ __device__ __forceinline__ void tp_merge_items(const TpOrder &o, int r, long lon
             long long lo = diag > nb ? diag - nb : 0, hi = diag < na ? diag : na;
             while (lo < hi) {
                 const long long mid = (lo + hi) >> 1;
-                if (key_cmp_words(o.key + o.key_off[in[a_lo + mid]] + skip,
-                                  o.key + o.key_off[in[a_hi + diag - mid - 1]] + skip, o.bits) <= 0)
+                if (key_cmp_words<BITS>(o.key + o.key_off[in[a_lo + mid]] + skip,
+                                        o.key + o.key_off[in[a_hi + diag - mid - 1]] + skip) <= 0)
                     lo = mid + 1;
                 else
                     hi = mid;
@@ -267,7 +267,7 @@ __device__ __forceinline__ void tp_merge_items(const TpOrder &o, int r, long lon
         if (i >= a_hi) take_a = false;
         else if (j >= b_hi) take_a = true;
         else if (wa != wb) take_a = wa < wb;
-        else take_a = key_end(wa, o.bits) || key_cmp_words(ka + 1, kb + 1, o.bits) <= 0;
+        else take_a = key_end<BITS>(wa) || key_cmp_words<BITS>(ka + 1, kb + 1) <= 0;
         out[d] = take_a ? ia : ib;
         if (take_a) {
             ++i;
@@ -281,11 +281,12 @@ __device__ __forceinline__ void tp_merge_items(const TpOrder &o, int r, long lon
 
 // the TP at position i differs from the one before it (TPs of different slots,
 // and of one sub-run, always do)
+template <int BITS>
 __device__ __forceinline__ bool tp_differs(const TpOrder &o, long long i) {
     const int4 info = o.sub_info[o.pos_sub[i]];
     if (info.y == 1 || i == o.bounds[info.x]) return true;
-    return key_cmp_words(o.key + o.key_off[o.perm[0][i - 1]] + info.z, o.key + o.key_off[o.perm[0][i]] + info.z,
-                         o.bits) != 0;
+    return key_cmp_words<BITS>(o.key + o.key_off[o.perm[0][i - 1]] + info.z,
+                               o.key + o.key_off[o.perm[0][i]] + info.z) != 0;
 }
 
 // TPs that a warp of the two kernels below takes at a time, of P: their parts
