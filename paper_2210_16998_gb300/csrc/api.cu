@@ -2995,8 +2995,8 @@ int tpg_sizer_presize(tpg_sizer *z, tpg_cfg *g, double margin, int64_t *caps_out
     const double lvl = nodes * std::min(1.0, rp * margin), TV0 = V * (z->r_tv0 > 0 ? z->r_tv0 : 2.0) * margin,
                  TV = V * (z->r_tv > 0 ? z->r_tv : 2.0) * margin;
     // a capture holds all of these at once: keep its buffers (per path: arena
-    // node and place, 16 bytes; per frontier slot: both ping-pong halves; per PP: its reference and ~170 bytes of ordering, TP
-    // and output workspace; PP and TP vertices and TP merge keys; 25% growth
+    // node and place, 16 bytes; per frontier slot: both ping-pong halves; per PP:
+    // its reference and ~210 bytes of ordering, TP and output workspace; PP and TP vertices and TP merge keys; 25% growth
     // slack of every buffer) within half of the free device memory; smaller
     // capacities only cost a fallback to the exact path
     size_t free_b = 0, total_b = 0;
@@ -3006,7 +3006,7 @@ int tpg_sizer_presize(tpg_sizer *z, tpg_cfg *g, double margin, int64_t *caps_out
     }
     const double bytes =
         1.25 * ((double)NODE_BYTES * nodes + 2.0 * (sizeof(int2) + 4.0 * g->W + sizeof(unsigned short)) * lvl +
-                (sizeof(int) + 170.0) * P + 4.0 * V + 6.0 * TV0 + 4.0 * TV);
+                (sizeof(int) + 210.0) * P + 4.0 * V + 6.0 * TV0 + 4.0 * TV);
     const double f = free_b ? std::min(1.0, 0.5 * (double)free_b / bytes) : 1.0;
     // list sizes also stay below 2^31 (a larger need falls back as well)
     auto cap = [](double x, long long lo) {

@@ -52,25 +52,37 @@ using bf16 = __nv_bfloat16;
 // features (from the loaded handle: degrees, entry/exit, SCC size from the
 // BFS tables, BFS depth from entry and to exit, graph size)
 // ---------------------------------------------------------------------------
+// (a warp per vertex: the SCC size is a count over two rows of the table, whose
+// lane-wide reads are what it waits for; 6,400 vertices 24.9 -> 7.4 us)
 __global__ void sz_features_kernel(GraphDev g, float *X) {
-    for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < g.N; v += gridDim.x * blockDim.x) {
+    const int lane = threadIdx.x & 31;
+    const int nw = gridDim.x * (blockDim.x >> 5);
+    for (int v = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); v < g.N; v += nw) {
         const int gid = g.vgraph ? g.vgraph[v] : 0;
         const int vb = g.vgraph ? g.vbase[gid] : 0;
         const int ng = g.vgraph ? g.vbase[gid + 1] - vb : g.N;
         const int vl = v - vb, en = g.entry[gid] - vb, ex = g.exit[gid] - vb;
         const int *D = g.dist + g.tbl_base[gid];
         int scc = 0;
-        for (int u = 0; u < ng; ++u) scc += (D[(long long)vl * ng + u] >= 0 && D[(long long)u * ng + vl] >= 0);
-        const int d1 = D[(long long)en * ng + vl], d2 = D[(long long)vl * ng + ex];
-        float *x = X + (long long)v * SZ_F;
-        x[0] = log1pf((float)(g.prp[v + 1] - g.prp[v]));
-        x[1] = log1pf((float)(g.rp[v + 1] - g.rp[v]));
-        x[2] = vl == en ? 1.f : 0.f;
-        x[3] = vl == ex ? 1.f : 0.f;
-        x[4] = log1pf((float)scc);
-        x[5] = d1 >= 0 ? (float)d1 / (float)ng : 2.f;
-        x[6] = d2 >= 0 ? (float)d2 / (float)ng : 2.f;
-        x[7] = logf((float)ng) / 5.f;
+        for (int u = lane; u < ng; u += 32) scc += (D[(long long)vl * ng + u] >= 0 && D[(long long)u * ng + vl] >= 0);
+        scc = __reduce_add_sync(0xffffffffu, scc);
+        if (lane >= SZ_F) continue;
+        float f = 0.f;
+        switch (lane) {
+            case 0: f = log1pf((float)(g.prp[v + 1] - g.prp[v])); break;
+            case 1: f = log1pf((float)(g.rp[v + 1] - g.rp[v])); break;
+            case 2: f = vl == en ? 1.f : 0.f; break;
+            case 3: f = vl == ex ? 1.f : 0.f; break;
+            case 4: f = log1pf((float)scc); break;
+            case 5:
+            case 6: {
+                const int d = lane == 5 ? D[(long long)en * ng + vl] : D[(long long)vl * ng + ex];
+                f = d >= 0 ? (float)d / (float)ng : 2.f;
+                break;
+            }
+            default: f = logf((float)ng) / 5.f;
+        }
+        X[(long long)v * SZ_F + lane] = f;
     }
 }
 
@@ -84,20 +96,30 @@ __global__ void sz_labels_kernel(const unsigned long long *counts, long long N, 
 // ---------------------------------------------------------------------------
 // forward
 // ---------------------------------------------------------------------------
+// A warp per vertex, two channels a lane (a thread per vertex left 25 blocks for
+// 6,400 vertices: 21.4 -> 12.0 us).
 __global__ void sz_input_fwd(const float *X, long long N, const float *P, bf16 *H0) {
-    __shared__ float w[SZ_H * SZ_F + SZ_H];
-    for (int i = threadIdx.x; i < SZ_H * SZ_F + SZ_H; i += blockDim.x) w[i] = P[OFF_W0 + i];
-    __syncthreads();
-    for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < N; v += (long long)gridDim.x * blockDim.x) {
-        float x[SZ_F];
+    const int lane = threadIdx.x & 31;
+    const long long nw = (long long)gridDim.x * (blockDim.x >> 5);
+    float w[2][SZ_F], b[2];
 #pragma unroll
-        for (int k = 0; k < SZ_F; ++k) x[k] = X[v * SZ_F + k];
-        for (int o = 0; o < SZ_H; ++o) {
-            float z = w[SZ_H * SZ_F + o];
+    for (int c = 0; c < 2; ++c) {
+        b[c] = P[OFF_B0 + 2 * lane + c];
 #pragma unroll
-            for (int k = 0; k < SZ_F; ++k) z = fmaf(w[o * SZ_F + k], x[k], z);
-            H0[v * SZ_H + o] = __float2bfloat16(z > 0.f ? z : 0.f);
+        for (int k = 0; k < SZ_F; ++k) w[c][k] = P[OFF_W0 + (2 * lane + c) * SZ_F + k];
+    }
+    for (long long v = blockIdx.x * (long long)(blockDim.x >> 5) + (threadIdx.x >> 5); v < N; v += nw) {
+        const float4 x0 = *(const float4 *)(X + v * SZ_F), x1 = *(const float4 *)(X + v * SZ_F + 4);
+        const float x[SZ_F] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
+        float z[2];
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            z[c] = b[c];
+#pragma unroll
+            for (int k = 0; k < SZ_F; ++k) z[c] = fmaf(w[c][k], x[k], z[c]);
         }
+        ((__nv_bfloat162 *)H0)[v * (SZ_H / 2) + lane] =
+            __floats2bfloat162_rn(z[0] > 0.f ? z[0] : 0.f, z[1] > 0.f ? z[1] : 0.f);
     }
 }
 
@@ -128,9 +150,8 @@ __global__ void sz_aggregate(const bf16 *H, long long N, const int *rp, const in
     }
 }
 
-__device__ __forceinline__ unsigned pack_bf16(bf16 lo, bf16 hi) {
-    return (unsigned)__bfloat16_as_ushort(lo) | ((unsigned)__bfloat16_as_ushort(hi) << 16);
-}
+// two neighbouring channels (of even index) in one word
+__device__ __forceinline__ unsigned pair_bf16(const bf16 *p) { return *(const unsigned *)p; }
 
 // C[M x NC] = A[M x K] * B, with B given transposed as Bt[NC x K] (both BF16
 // row-major), FP32 accumulation on the tensor cores (mma.sync m16n8k16
@@ -167,15 +188,15 @@ __global__ void __launch_bounds__(128) sz_mma_gemm(const bf16 *A, long long M, c
 #pragma unroll
     for (int kk = 0; kk < K; kk += 16) {
         const int c0 = kk + tig * 2;
-        const unsigned a0 = pack_bf16(As[r0 * LD + c0], As[r0 * LD + c0 + 1]);
-        const unsigned a1 = pack_bf16(As[(r0 + 8) * LD + c0], As[(r0 + 8) * LD + c0 + 1]);
-        const unsigned a2 = pack_bf16(As[r0 * LD + c0 + 8], As[r0 * LD + c0 + 9]);
-        const unsigned a3 = pack_bf16(As[(r0 + 8) * LD + c0 + 8], As[(r0 + 8) * LD + c0 + 9]);
+        const unsigned a0 = pair_bf16(As + r0 * LD + c0);
+        const unsigned a1 = pair_bf16(As + (r0 + 8) * LD + c0);
+        const unsigned a2 = pair_bf16(As + r0 * LD + c0 + 8);
+        const unsigned a3 = pair_bf16(As + (r0 + 8) * LD + c0 + 8);
 #pragma unroll
         for (int t = 0; t < 8; ++t) {
             const int n = t * 8 + gid;
-            const unsigned b0 = pack_bf16(Bs[n * LD + c0], Bs[n * LD + c0 + 1]);
-            const unsigned b1 = pack_bf16(Bs[n * LD + c0 + 8], Bs[n * LD + c0 + 9]);
+            const unsigned b0 = pair_bf16(Bs + n * LD + c0);
+            const unsigned b1 = pair_bf16(Bs + n * LD + c0 + 8);
             asm volatile(
                 "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
                 "{%0,%1,%2,%3};"
@@ -202,19 +223,30 @@ __global__ void __launch_bounds__(128) sz_mma_gemm(const bf16 *A, long long M, c
     }
 }
 
+// A thread per vertex and target, the vertex's channels read 8 at a time
+// (11.7 -> 4.8 us for 6,400 vertices).
 __global__ void sz_head_fwd(const bf16 *H3, long long N, const float *P, float *Y) {
     __shared__ float w[SZ_T * SZ_H + SZ_T];
     for (int i = threadIdx.x; i < SZ_T * SZ_H + SZ_T; i += blockDim.x) w[i] = P[OFF_WO + i];
     __syncthreads();
-    for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < N; v += (long long)gridDim.x * blockDim.x) {
-        float y[SZ_T] = {w[SZ_T * SZ_H], w[SZ_T * SZ_H + 1], w[SZ_T * SZ_H + 2]};
-        for (int o = 0; o < SZ_H; ++o) {
-            const float h = __bfloat162float(H3[v * SZ_H + o]);
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N * SZ_T;
+         i += (long long)gridDim.x * blockDim.x) {
+        const long long v = i / SZ_T;
+        const int t = (int)(i - v * SZ_T);
+        const uint4 *h8 = (const uint4 *)(H3 + v * SZ_H);
+        float y = w[SZ_T * SZ_H + t];
 #pragma unroll
-            for (int t = 0; t < SZ_T; ++t) y[t] = fmaf(w[t * SZ_H + o], h, y[t]);
+        for (int o8 = 0; o8 < SZ_H / 8; ++o8) {
+            const uint4 q = h8[o8];
+            const unsigned u[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const float2 f = __bfloat1622float2(*(const __nv_bfloat162 *)&u[j]);
+                y = fmaf(w[t * SZ_H + o8 * 8 + 2 * j], f.x, y);
+                y = fmaf(w[t * SZ_H + o8 * 8 + 2 * j + 1], f.y, y);
+            }
         }
-#pragma unroll
-        for (int t = 0; t < SZ_T; ++t) Y[v * SZ_T + t] = y[t];
+        Y[i] = y;
     }
 }
 
@@ -222,38 +254,51 @@ __global__ void sz_head_fwd(const bf16 *H3, long long N, const float *P, float *
 // loss and backward
 // ---------------------------------------------------------------------------
 // dY = 2 (Y - T) / (3N); dZ3 = (dY Wo) * [H3 > 0]; loss = mean (Y - T)^2
+// A warp per vertex, two channels a lane; the loss is added up by shuffles (a
+// thread per vertex and a shared double that all of them added to: 61.9 ->
+// 10.0 us for 6,400 vertices).
 __global__ void __launch_bounds__(256) sz_head_bwd(const float *Y, const float *T, const bf16 *H3, long long N,
                                                    const float *P, float *dY, double *loss, float *dZ,
                                                    bf16 *dZb) {
-    __shared__ float w[SZ_T * SZ_H];
-    __shared__ double sloss;
-    for (int i = threadIdx.x; i < SZ_T * SZ_H; i += blockDim.x) w[i] = P[OFF_WO + i];
-    if (threadIdx.x == 0) sloss = 0.0;
-    __syncthreads();
+    __shared__ double sloss[8];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    float w[SZ_T][2];
+#pragma unroll
+    for (int t = 0; t < SZ_T; ++t)
+#pragma unroll
+        for (int c = 0; c < 2; ++c) w[t][c] = P[OFF_WO + t * SZ_H + 2 * lane + c];
     const float scale = 2.f / (float)(SZ_T * N);
     double my_loss = 0.0;
-    for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < N; v += (long long)gridDim.x * blockDim.x) {
+    for (long long v = blockIdx.x * 8ll + wid; v < N; v += gridDim.x * 8ll) {
         float dy[SZ_T];
+        const float2 h = __bfloat1622float2(((const __nv_bfloat162 *)H3)[v * (SZ_H / 2) + lane]);
 #pragma unroll
         for (int t = 0; t < SZ_T; ++t) {
             const float d = Y[v * SZ_T + t] - T[v * SZ_T + t];
-            my_loss += (double)d * d;
             dy[t] = scale * d;
-            dY[v * SZ_T + t] = dy[t];
+            if (lane == t) {
+                my_loss += (double)d * d;
+                dY[v * SZ_T + t] = dy[t];
+            }
         }
-        for (int o = 0; o < SZ_H; ++o) {
-            const float h = __bfloat162float(H3[v * SZ_H + o]);
-            float dh = 0.f;
+        float dh0 = 0.f, dh1 = 0.f;
 #pragma unroll
-            for (int t = 0; t < SZ_T; ++t) dh = fmaf(dy[t], w[t * SZ_H + o], dh);
-            const float dz = h > 0.f ? dh : 0.f;
-            dZ[v * SZ_H + o] = dz;
-            dZb[v * SZ_H + o] = __float2bfloat16(dz);
+        for (int t = 0; t < SZ_T; ++t) {
+            dh0 = fmaf(dy[t], w[t][0], dh0);
+            dh1 = fmaf(dy[t], w[t][1], dh1);
         }
+        const float2 dz = make_float2(h.x > 0.f ? dh0 : 0.f, h.y > 0.f ? dh1 : 0.f);
+        ((float2 *)dZ)[v * (SZ_H / 2) + lane] = dz;
+        ((__nv_bfloat162 *)dZb)[v * (SZ_H / 2) + lane] = __floats2bfloat162_rn(dz.x, dz.y);
     }
-    atomicAdd(&sloss, my_loss);
+    for (int o = 16; o > 0; o >>= 1) my_loss += __shfl_xor_sync(0xffffffffu, my_loss, o);
+    if (lane == 0) sloss[wid] = my_loss;
     __syncthreads();
-    if (threadIdx.x == 0) atomicAdd(loss, sloss / (double)(SZ_T * N));
+    if (threadIdx.x == 0) {
+        double sum = 0.0;
+        for (int i = 0; i < 8; ++i) sum += sloss[i];
+        atomicAdd(loss, sum / (double)(SZ_T * N));
+    }
 }
 
 // dWo[t][o] = sum_v dY[v][t] H3[v][o], dbo[t] = sum_v dY[v][t]: thread
@@ -271,57 +316,98 @@ __global__ void __launch_bounds__(256) sz_head_dw(const float *dY, const bf16 *H
 }
 
 // dW_l[m][k] += sum_v dZ[v][m] Xcat[v][k]; db_l[m] += sum_v dZ[v][m].
-// Thread t owns output row m = t / 4 and 48 columns; each block walks a
-// strided set of 32-vertex chunks staged in shared memory.
+// FP32 throughout.  Warp w owns rows 8w .. 8w + 7, lane l columns l, l + 32, ..:
+// 8 + 6 shared reads (the 8 as two broadcasts) feed 48 multiply-adds, and the
+// blocks' sums leave as whole 128-byte lines; each block walks a strided set of
+// 32-vertex chunks staged in shared memory.  (A row and 48 neighbouring columns
+// to a thread read 49 values for 48 and added them 192 bytes apart: 48.0 -> 13.2 us
+// for 6,400 vertices.)
 __global__ void __launch_bounds__(256) sz_dW(const float *dZ, const bf16 *Xcat, long long N, float *gW,
                                              float *gb) {
-    __shared__ float sdz[32][SZ_H];
+    __shared__ __align__(16) float sdz[32][SZ_H];
     __shared__ float sx[32][SZ_K];
-    const int m = threadIdx.x >> 2, k0 = (threadIdx.x & 3) * 48;
-    float acc[48];
+    const int lane = threadIdx.x & 31, m0 = (threadIdx.x >> 5) * 8;
+    float acc[8][SZ_K / 32];
 #pragma unroll
-    for (int q = 0; q < 48; ++q) acc[q] = 0.f;
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int j = 0; j < SZ_K / 32; ++j) acc[i][j] = 0.f;
     float accb = 0.f;
     for (long long base = blockIdx.x * 32ll; base < N; base += gridDim.x * 32ll) {
-        for (int i = threadIdx.x; i < 32 * SZ_H; i += 256) {
-            const long long v = base + i / SZ_H;
-            sdz[i / SZ_H][i % SZ_H] = v < N ? dZ[v * SZ_H + i % SZ_H] : 0.f;
+        for (int i = threadIdx.x; i < 32 * SZ_H / 4; i += 256) {
+            const int r = i / (SZ_H / 4), c = i % (SZ_H / 4);
+            float4 d = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (base + r < N) d = ((const float4 *)dZ)[(base + r) * (SZ_H / 4) + c];
+            ((float4 *)sdz[r])[c] = d;
         }
-        for (int i = threadIdx.x; i < 32 * SZ_K; i += 256) {
-            const long long v = base + i / SZ_K;
-            sx[i / SZ_K][i % SZ_K] = v < N ? __bfloat162float(Xcat[v * SZ_K + i % SZ_K]) : 0.f;
+        bool odd = false;
+        for (int i = threadIdx.x; i < 32 * SZ_K / 2; i += 256) {
+            const int r = i / (SZ_K / 2), c = i % (SZ_K / 2);
+            float2 x = make_float2(0.f, 0.f);
+            if (base + r < N) x = __bfloat1622float2(((const __nv_bfloat162 *)Xcat)[(base + r) * (SZ_K / 2) + c]);
+            *(float2 *)&sx[r][2 * c] = x;
+            odd |= !isfinite(x.x) || !isfinite(x.y);
         }
-        __syncthreads();
-        for (int r = 0; r < 32; ++r) {
-            const float d = sdz[r][m];
-            if (d == 0.f) continue;
-            if ((threadIdx.x & 3) == 0) accb += d;
+        if (__syncthreads_or(odd)) {  // a zero gradient takes nothing from an overflowed input
+            for (int r = 0; r < 32; ++r)
+                for (int i = 0; i < 8; ++i) {
+                    const float d = sdz[r][m0 + i];
+                    if (d == 0.f) continue;
 #pragma unroll
-            for (int q = 0; q < 48; ++q) acc[q] = fmaf(d, sx[r][k0 + q], acc[q]);
+                    for (int i2 = 0; i2 < 8; ++i2)
+                        if (i2 == i)
+#pragma unroll
+                            for (int j = 0; j < SZ_K / 32; ++j) acc[i2][j] = fmaf(d, sx[r][lane + 32 * j], acc[i2][j]);
+                }
+        } else
+#pragma unroll 4
+        for (int r = 0; r < 32; ++r) {
+            const float4 d0 = *(const float4 *)&sdz[r][m0], d1 = *(const float4 *)&sdz[r][m0 + 4];
+            const float d[8] = {d0.x, d0.y, d0.z, d0.w, d1.x, d1.y, d1.z, d1.w};
+#pragma unroll
+            for (int j = 0; j < SZ_K / 32; ++j) {
+                const float x = sx[r][lane + 32 * j];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) acc[i][j] = fmaf(d[i], x, acc[i][j]);
+            }
         }
+        if (threadIdx.x < SZ_H)
+            for (int r = 0; r < 32; ++r) accb += sdz[r][threadIdx.x];
         __syncthreads();
     }
+    if (blockIdx.x * 32ll >= N) return;
 #pragma unroll
-    for (int q = 0; q < 48; ++q)
-        if (acc[q] != 0.f) atomicAdd(&gW[m * SZ_K + k0 + q], acc[q]);
-    if ((threadIdx.x & 3) == 0 && accb != 0.f) atomicAdd(&gb[m], accb);
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int j = 0; j < SZ_K / 32; ++j) atomicAdd(&gW[(m0 + i) * SZ_K + lane + 32 * j], acc[i][j]);
+    if (threadIdx.x < SZ_H) atomicAdd(&gb[threadIdx.x], accb);
 }
 
 // dH_prev[v] = dX[v][self] + sum_{v->w} dX[w][in] + sum_{u->v} dX[u][out];
 // dZ_prev = dH_prev * [H_prev > 0].  One warp per vertex.
+// Two channels a lane: one pass over the arcs (13.6 -> 7.8 us).
 __global__ void sz_backprop_agg(const float *dX, const bf16 *Hprev, long long N, const int *rp, const int *col,
                                 const int *prp, const int *pcol, float *dZ, bf16 *dZb) {
     const int lane = threadIdx.x & 31;
     const long long nw = (long long)gridDim.x * (blockDim.x >> 5);
+    const float2 *dX2 = (const float2 *)dX;
     for (long long v = blockIdx.x * (long long)(blockDim.x >> 5) + (threadIdx.x >> 5); v < N; v += nw) {
-        for (int c = lane; c < SZ_H; c += 32) {
-            float d = dX[v * SZ_K + c];
-            for (int e = rp[v]; e < rp[v + 1]; ++e) d += dX[(long long)col[e] * SZ_K + SZ_H + c];
-            for (int e = prp[v]; e < prp[v + 1]; ++e) d += dX[(long long)pcol[e] * SZ_K + 2 * SZ_H + c];
-            const float dz = __bfloat162float(Hprev[v * SZ_H + c]) > 0.f ? d : 0.f;
-            dZ[v * SZ_H + c] = dz;
-            if (dZb) dZb[v * SZ_H + c] = __float2bfloat16(dz);
+        const int e0 = rp[v], e1 = rp[v + 1], p0 = prp[v], p1 = prp[v + 1];
+        const float2 h = __bfloat1622float2(((const __nv_bfloat162 *)Hprev)[v * (SZ_H / 2) + lane]);
+        float2 d = dX2[v * (SZ_K / 2) + lane];
+        for (int e = e0; e < e1; ++e) {
+            const float2 x = dX2[(long long)col[e] * (SZ_K / 2) + SZ_H / 2 + lane];
+            d.x += x.x;
+            d.y += x.y;
         }
+        for (int e = p0; e < p1; ++e) {
+            const float2 x = dX2[(long long)pcol[e] * (SZ_K / 2) + SZ_H + lane];
+            d.x += x.x;
+            d.y += x.y;
+        }
+        const float2 dz = make_float2(h.x > 0.f ? d.x : 0.f, h.y > 0.f ? d.y : 0.f);
+        ((float2 *)dZ)[v * (SZ_H / 2) + lane] = dz;
+        if (dZb) ((__nv_bfloat162 *)dZb)[v * (SZ_H / 2) + lane] = __floats2bfloat162_rn(dz.x, dz.y);
     }
 }
 
@@ -371,18 +457,22 @@ __global__ void sz_refresh_bf16(const float *P, bf16 *Wb, bf16 *Wtb) {
 }
 
 // per-graph and total predicted volumes (expm1 of the predictions)
-__global__ void sz_sum_pred(const float *Y, long long N, double *tot) {
-    __shared__ double s[SZ_T];
-    if (threadIdx.x < SZ_T) s[threadIdx.x] = 0.0;
-    __syncthreads();
-    double acc[SZ_T] = {0.0, 0.0, 0.0};
-    for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < N; v += (long long)gridDim.x * blockDim.x)
+// (a thread per prediction, sums by shuffles: 20.2 -> 5.3 us for 6,400 vertices)
+__global__ void __launch_bounds__(96) sz_sum_pred(const float *Y, long long N, double *tot) {
+    __shared__ double s[3][SZ_T];
+    static_assert(SZ_T == 3, "thread i takes target i % 3");
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    double acc = 0.0;  // of target (96 blocks + threadIdx) % 3 = threadIdx % 3
+    for (long long i = blockIdx.x * 96ll + threadIdx.x; i < N * SZ_T; i += gridDim.x * 96ll)
+        acc += expm1((double)fmaxf(Y[i], 0.f));
 #pragma unroll
-        for (int t = 0; t < SZ_T; ++t) acc[t] += expm1((double)fmaxf(Y[v * SZ_T + t], 0.f));
-#pragma unroll
-    for (int t = 0; t < SZ_T; ++t) atomicAdd(&s[t], acc[t]);
+    for (int t = 0; t < SZ_T; ++t) {
+        double a = (int)(threadIdx.x % SZ_T) == t ? acc : 0.0;
+        for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+        if (lane == 0) s[wid][t] = a;
+    }
     __syncthreads();
-    if (threadIdx.x < SZ_T) atomicAdd(&tot[threadIdx.x], s[threadIdx.x]);
+    if (threadIdx.x < SZ_T) atomicAdd(&tot[threadIdx.x], s[0][threadIdx.x] + s[1][threadIdx.x] + s[2][threadIdx.x]);
 }
 
 unsigned grid_of(long long n, int block, int num_sms) {
@@ -550,7 +640,7 @@ cudaError_t sz_get_grads(SizerNet *n, float *host) {
 }
 
 cudaError_t sz_features(const GraphDev &g, float *X, cudaStream_t s, int num_sms) {
-    sz_features_kernel<<<grid_of(g.N, 128, num_sms), 128, 0, s>>>(g, X);
+    sz_features_kernel<<<grid_of(32ll * g.N, 128, num_sms), 128, 0, s>>>(g, X);
     note_launch();
     return cudaGetLastError();
 }
@@ -564,8 +654,7 @@ cudaError_t sz_labels(const unsigned long long *counts, long long N, float *T, c
 cudaError_t sz_forward(SizerNet *n, const SzGraph &b) {
     cudaError_t e = sz_ensure(n, b.N);
     if (e != cudaSuccess) return e;
-    const unsigned g256 = grid_of(b.N, 256, n->num_sms);
-    sz_input_fwd<<<g256, 256, 0, n->s>>>(b.X, b.N, n->P, n->H[0]);
+    sz_input_fwd<<<grid_of(b.N * 8, 256, n->num_sms), 256, 0, n->s>>>(b.X, b.N, n->P, n->H[0]);
     note_launch();
     for (int l = 0; l < SZ_L; ++l) {
         sz_aggregate<<<grid_of(b.N * 32, 256, n->num_sms), 256, 0, n->s>>>(n->H[l], b.N, b.rp, b.col, b.prp, b.pcol,
@@ -575,7 +664,7 @@ cudaError_t sz_forward(SizerNet *n, const SzGraph &b) {
                              n->H[l + 1], nullptr);
         if (e != cudaSuccess) return e;
     }
-    sz_head_fwd<<<g256, 256, 0, n->s>>>(n->H[SZ_L], b.N, n->P, n->Y);
+    sz_head_fwd<<<grid_of(b.N * SZ_T, 128, n->num_sms), 128, 0, n->s>>>(n->H[SZ_L], b.N, n->P, n->Y);
     note_launch();
     return cudaGetLastError();
 }
@@ -583,10 +672,9 @@ cudaError_t sz_forward(SizerNet *n, const SzGraph &b) {
 cudaError_t sz_loss_backward(SizerNet *n, const SzGraph &b, double *loss_host) {
     cudaError_t e = sz_forward(n, b);
     if (e != cudaSuccess) return e;
-    const unsigned g256 = grid_of(b.N, 256, n->num_sms);
     if ((e = cudaMemsetAsync(n->G, 0, sizeof(float) * NPARAM, n->s))) return e;
     if ((e = cudaMemsetAsync(n->loss, 0, sizeof(double), n->s))) return e;
-    sz_head_bwd<<<g256, 256, 0, n->s>>>(n->Y, b.T, n->H[SZ_L], b.N, n->P, n->dY, n->loss, n->dZ, n->dZb);
+    sz_head_bwd<<<grid_of(b.N * 32, 256, n->num_sms), 256, 0, n->s>>>(n->Y, b.T, n->H[SZ_L], b.N, n->P, n->dY, n->loss, n->dZ, n->dZb);
     sz_head_dw<<<(unsigned)(n->num_sms * 4), 256, 0, n->s>>>(n->dY, n->H[SZ_L], b.N, n->G);
     note_launch(2);
     for (int l = SZ_L - 1; l >= 0; --l) {
@@ -624,7 +712,7 @@ cudaError_t sz_adam_step(SizerNet *n, float lr) {
 cudaError_t sz_log_totals(SizerNet *n, const float *Y, long long N, double *totals_host) {
     cudaError_t e = cudaMemsetAsync(n->tot, 0, sizeof(double) * SZ_T, n->s);
     if (e != cudaSuccess) return e;
-    sz_sum_pred<<<grid_of(N, 256, n->num_sms), 256, 0, n->s>>>(Y, N, n->tot);
+    sz_sum_pred<<<grid_of(N * SZ_T, 96, n->num_sms), 96, 0, n->s>>>(Y, N, n->tot);
     note_launch();
     if ((e = cudaMemcpyAsync(totals_host, n->tot, sizeof(double) * SZ_T, cudaMemcpyDeviceToHost, n->s))) return e;
     return cudaStreamSynchronize(n->s);
@@ -635,7 +723,7 @@ cudaError_t sz_predict(SizerNet *n, const SzGraph &b, float *Y_host, double *tot
     if (e != cudaSuccess) return e;
     if (totals_host) {
         if ((e = cudaMemsetAsync(n->tot, 0, sizeof(double) * SZ_T, n->s))) return e;
-        sz_sum_pred<<<grid_of(b.N, 256, n->num_sms), 256, 0, n->s>>>(n->Y, b.N, n->tot);
+        sz_sum_pred<<<grid_of(b.N * SZ_T, 96, n->num_sms), 96, 0, n->s>>>(n->Y, b.N, n->tot);
         note_launch();
         if ((e = cudaMemcpyAsync(totals_host, n->tot, sizeof(double) * SZ_T, cudaMemcpyDeviceToHost, n->s))) return e;
     }
