@@ -1330,12 +1330,113 @@ int tp_order_arrays(tpg_cfg *g, DevBuf &subs_buf, DevBuf &slots_buf, long long s
 // ---------------------------------------------------------------------------
 // test paths
 // ---------------------------------------------------------------------------
+// Lists this short are made by one block (tp_small): most PPs, and most
+// vertices a list of them can have (the room for it is the upper bound).  The
+// whole call, general path -> one block: 102 PPs 194 -> 41 us, 1116 215 -> 67,
+// 2075 214 -> 103, 4558 250 -> 205, 6519 216 -> 189, 8860 251 -> 304; chains of
+// 300, 1000, 1500 vertices 337 -> 115, 695 -> 524, 930 -> 933.
+constexpr long long TP_SMALL_P = 4096, TP_SMALL_V = 1 << 21;
+
+bool tp_is_small(const tpg_cfg *g) {
+    return g->G == 1 && g->P > 0 && g->P <= TP_SMALL_P && g->V + 2ll * g->maxn * g->P <= TP_SMALL_V;
+}
+
+int run_test_paths_small(tpg_cfg *g, Block **o_off, Block **o_vert, Block **o_gptr, long long *oT, long long *oTV,
+                         int *pp_to_tp) {
+    cudaStream_t s = g->stream;
+    const long long P = g->P, V_ub = g->V + 2ll * g->maxn * P;
+    const int kbits = g->maxn <= 255 ? 8 : 16;
+    TpSmallArgs a{};
+    RC(ensure(g, g->s_i64[0], sizeof(long long) * (P + 1)));
+    RC(ensure(g, g->s_i64[1], sizeof(long long) * (P + 1)));
+    RC(ensure(g, g->s_i64[2], sizeof(long long) * (P + 1)));
+    RC(ensure(g, g->s_i32[0], sizeof(int) * (P + 1)));
+    RC(ensure(g, g->s_i32[1], sizeof(int) * (P + 1)));
+    RC(ensure(g, g->s_i32[2], sizeof(int) * (P + 1)));
+    RC(ensure(g, g->s_refs[0], sizeof(long long) * (P + 1)));
+    RC(ensure(g, g->s_refs[1], sizeof(long long) * (P + 1)));
+    RC(ensure(g, g->tp_key_off, sizeof(long long) * (P + 1)));
+    RC(ensure(g, g->tp_key, sizeof(unsigned long long) * (V_ub / (64 / kbits) + P + KEY_PAD)));
+    RC(ensure(g, g->ctl, CTL_BYTES));
+    RC(tp_order_arrays(g, g->tp_subs, g->tp_slots, P, &a.o));
+    Block *off = block_new(g->fns, sizeof(long long) * (P + 1), s);
+    Block *vert = block_new(g->fns, sizeof(int) * V_ub, s);
+    Block *gptr = block_new(g->fns, sizeof(long long) * 2, s);
+    int rc = off && vert && gptr ? TPG_OK : TPG_ENOMEM;
+    long long *h = (long long *)g->h_small;
+    if (rc == TPG_OK) {
+        a.o.pp_off = (const long long *)g->pp_off->p;
+        a.o.pp_vert = (const int *)g->pp_vert->p;
+        a.o.start = g->s_i32[0].as<int>();
+        a.o.pos_sub = g->s_i32[1].as<int>();
+        a.o.sub_rank = g->s_i64[1].as<long long>();
+        a.o.perm[0] = g->s_refs[0].as<long long>();
+        a.o.perm[1] = g->s_refs[1].as<long long>();
+        a.o.key_off = a.key_off = g->tp_key_off.as<long long>();
+        a.o.key = a.key = g->tp_key.as<unsigned long long>();
+        a.o.bits = kbits;
+        a.P = P;
+        a.V = g->V;
+        a.slots = g->M + g->N;
+        a.ends = g->pp_ends.as<int2>();
+        a.tp_len = g->s_i64[0].as<long long>();
+        a.tp_off = g->s_i64[2].as<long long>();
+        a.keep = a.o.start;          // the starts are used up by then
+        a.keep_off = a.o.sub_rank;   // and so are the ranks
+        a.keep_rank = a.o.perm[1];
+        a.out_graph = g->s_i32[2].as<int>();
+        a.final_off = (long long *)off->p;
+        a.out_vert = (int *)vert->p;
+        a.gptr = (long long *)gptr->p;
+        a.pp_to_tp = pp_to_tp;
+        a.result = g->ctl.as<long long>();
+        cudaEventRecord(g->ev[4], s);
+        if (cuda_err(tp_small(a, s)) ||
+            cuda_err(cudaMemcpyAsync(h, a.result, 4 * sizeof(long long), cudaMemcpyDeviceToHost, s)))
+            rc = TPG_ECUDA;
+        cudaEventRecord(g->ev[5], s);
+        if (cudaStreamSynchronize(s) != cudaSuccess && rc == TPG_OK) rc = TPG_ECUDA;
+    }
+    if (rc == TPG_OK && (h[0] & ERR_UNREACH)) rc = TPG_EUNREACH;
+    if (rc == TPG_OK) {
+        g->last_tv0 = h[1];
+        *oT = h[2];
+        *oTV = h[3];
+        if (h[1] == g->V) {  // every TP is its PP: the PP list's blocks serve both
+            block_unref(off);
+            block_unref(vert);
+            block_unref(gptr);
+            off = g->pp_off;
+            vert = g->pp_vert;
+            gptr = g->pp_gptr;
+            for (Block *b : {off, vert, gptr}) block_ref(b);
+            *oT = P;
+            *oTV = g->V;
+            if (pp_to_tp && (cuda_err(tp_index_map(nullptr, nullptr, nullptr, P, pp_to_tp, s)) ||
+                             cudaStreamSynchronize(s) != cudaSuccess))
+                rc = TPG_ECUDA;
+        }
+    }
+    if (rc != TPG_OK) {
+        for (Block *b : {off, vert, gptr}) block_unref(b);
+        return rc;
+    }
+    cudaEventElapsedTime(&g->stats.t_test_paths_ms, g->ev[4], g->ev[5]);
+    *o_off = off;
+    *o_vert = vert;
+    *o_gptr = gptr;
+    g->stats.test_paths = *oT;
+    g->stats.tp_vertices = *oTV;
+    return TPG_OK;
+}
+
 // pp_to_tp (optional, device int[P]) receives the index in the returned list
 // of every PP's TP(p).
 int run_test_paths(tpg_cfg *g, Block **o_off, Block **o_vert, Block **o_gptr, long long *oT, long long *oTV,
                    int *pp_to_tp = nullptr) {
     cudaStream_t s = g->stream;
     if (!g->pp_valid) RC(run_prime_paths(g));
+    if (tp_is_small(g)) return run_test_paths_small(g, o_off, o_vert, o_gptr, oT, oTV, pp_to_tp);
     const long long P = g->P;
     const int *pp_graph = g->pp_graph ? (const int *)g->pp_graph->p : nullptr;
     const long long *pp_off = (const long long *)g->pp_off->p;

@@ -372,6 +372,103 @@ cudaError_t tp_assemble(const TpOrder &o, const long long *keep_off, const long 
     return cudaGetLastError();
 }
 
+// ---------------------------------------------------------------------------
+// few TPs of one graph: lengths, order, keys, merging and lists in one block.
+// What bounds the steps above for such a list is that there are 25 launches and
+// two read-backs of them (76 TPs: the whole call 205 us); here a step costs a
+// block barrier and its own chain of loads (24 us, the whole call 44).
+// ---------------------------------------------------------------------------
+constexpr int TPS_BLOCK = 1024;
+
+// out[0 .. n] = exclusive prefix of f(0 .. n - 1), the total returned; all threads, a barrier at the end
+template <typename F>
+__device__ __forceinline__ long long tps_scan(long long n, long long *out, F f) {
+    long long carry = 0;
+    for (long long base = 0; base < n; base += TPS_BLOCK) {
+        const long long i = base + threadIdx.x;
+        long long total;
+        const long long ex = block_excl_scan_i64<TPS_BLOCK>(i < n ? (long long)f(i) : 0ll, total);
+        if (i < n) out[i] = carry + ex;
+        carry += total;
+    }
+    if (threadIdx.x == 0) out[n] = carry;
+    __syncthreads();
+    return carry;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(TPS_BLOCK) tp_small_kernel(TpSmallArgs a) {
+    constexpr int BITS = 8 * sizeof(T);
+    __shared__ int s_err;
+    const TpOrder &o = a.o;
+    const GraphDev &g = o.g;
+    const long long P = a.P, tid = threadIdx.x;
+    if (tid == 0) s_err = 0;
+    __syncthreads();
+    const long long TV = tps_scan(P, a.tp_off, [&](long long i) {
+        const int2 e = a.ends[i];
+        const int pl = g.pre_len[e.x], sl = g.suf_len[e.y];
+        if (pl == 0 || sl == 0) s_err = ERR_UNREACH;
+        const long long len = pl == 0 || sl == 0 ? 0 : (long long)(pl - 1) + (o.pp_off[i + 1] - o.pp_off[i]) + (sl - 1);
+        a.tp_len[i] = len;
+        return len;
+    });
+    if (s_err || TV == a.V) {  // (equal: every TP is its PP)
+        if (tid == 0) {
+            a.result[0] = s_err;
+            a.result[1] = TV;
+        }
+        return;
+    }
+    for (long long i = tid; i <= a.slots; i += TPS_BLOCK) o.slot_n[i] = 0;  // and max_k
+    tps_scan(P, a.key_off, [&](long long i) { return key_words(a.tp_len[i], BITS); });
+    tp_mark_subs(o, P, tid, TPS_BLOCK);
+    __syncthreads();
+    tps_scan(P, o.sub_rank, [&](long long i) { return o.start[i]; });
+    tp_list_subs(o, P, tid, TPS_BLOCK);
+    __syncthreads();
+    tp_count_subs(o, P, tid, TPS_BLOCK);
+    __syncthreads();
+    tps_scan(a.slots, o.slot_at, [&](long long i) { return o.slot_n[i]; });
+    tp_place_subs(o, P, tid, TPS_BLOCK);
+    __syncthreads();
+    tp_place(o, P, tid, TPS_BLOCK);
+    constexpr int WARPS = TPS_BLOCK / 32;
+    const long long each = ((P + WARPS - 1) / WARPS + 1) & ~1ll;
+    const int group = each < 32 ? (int)each : 32;
+    for (long long i0 = (tid >> 5) * group; i0 < P; i0 += WARPS * group)
+        tp_write_keys_warp<T>(o, a.tp_off, a.key, i0, group, P);
+    __syncthreads();
+    const int max_k = *(volatile int *)o.max_k;
+    for (int r = 0; 1 << r < max_k; ++r) {
+        for (long long d0 = tid; d0 < P; d0 += TPS_BLOCK) tp_merge_items<1, BITS>(o, r, P, d0);
+        __syncthreads();
+    }
+    const long long kept = tps_scan(P, a.keep_rank, [&](long long i) { return a.keep[i] = tp_differs<BITS>(o, i); });
+    const long long FTV = tps_scan(P, a.keep_off, [&](long long i) { return a.keep[i] ? a.tp_len[o.perm[0][i]] : 0ll; });
+    for (long long i0 = (tid >> 5) * group; i0 < P; i0 += WARPS * group)
+        tp_unpack_warp<T>(o, a.keep_off, a.keep_rank, a.final_off, a.out_vert, a.out_graph, i0, group, P);
+    if (a.pp_to_tp)
+        for (long long i = tid; i < P; i += TPS_BLOCK)
+            a.pp_to_tp[o.perm[0][i]] = (int)(a.keep[i] ? a.keep_rank[i] : a.keep_rank[i] - 1);
+    if (tid == 0) {
+        a.final_off[kept] = FTV;
+        a.gptr[0] = 0;
+        a.gptr[1] = kept;
+        a.result[0] = 0;
+        a.result[1] = TV;
+        a.result[2] = kept;
+        a.result[3] = FTV;
+    }
+}
+
+cudaError_t tp_small(const TpSmallArgs &a, cudaStream_t s) {
+    if (a.o.bits == 8) tp_small_kernel<unsigned char><<<1, TPS_BLOCK, 0, s>>>(a);
+    else tp_small_kernel<unsigned short><<<1, TPS_BLOCK, 0, s>>>(a);
+    note_launch();
+    return cudaGetLastError();
+}
+
 // one warp per kept TP: copy into its final slot
 __global__ void tp_gather_kernel(const long long *perm, const int *keep, const long long *keep_rank, long long P,
                                  const long long *off, const int *vert, const int *graph,

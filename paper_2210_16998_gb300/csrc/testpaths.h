@@ -47,4 +47,24 @@ cudaError_t tp_assemble(const TpOrder &o, const long long *keep_off, const long 
 cudaError_t tp_index_map(const long long *perm, const int *keep, const long long *keep_rank, long long P, int *map,
                          cudaStream_t s);
 
+// The whole of it for P TPs (P > 0) of one graph, in one block: result = {error
+// word, TP vertices before dedup, TPs, their vertices}, the last two and all
+// lists only if the first is 0 and the second is not V (the PPs' vertices).
+// o as for the steps above, with room for P sub-runs; final_off[P + 1],
+// out_vert for the vertices before dedup, pp_to_tp (tp_index_map) may be null.
+struct TpSmallArgs {
+    TpOrder o;
+    long long P, V, slots;
+    const int2 *ends;
+    long long *tp_len, *tp_off, *key_off, *keep_off, *keep_rank;
+    int *keep;
+    unsigned long long *key;
+    long long *final_off;
+    int *out_vert, *out_graph;
+    long long *gptr;
+    int *pp_to_tp;
+    long long *result;
+};
+cudaError_t tp_small(const TpSmallArgs &a, cudaStream_t s);
+
 }  // namespace tpg

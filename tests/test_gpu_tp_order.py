@@ -30,6 +30,7 @@ def lead_and_loops(lead, loops, size, skip):
 
 
 CASES = [(lead, loops, size, skip) for lead in (1, 5, 6, 7, 8, 9, 16) for loops, size, skip in ((1, 3, 1), (3, 6, 2))]
+CASES += [(2, loops, 5, 3) for loops in (6, 7, 8)]  # PPs below and above what one block takes
 CASES += [(3, 2, 40, 7), (235, 3, 6, 2), (236, 3, 6, 2), (237, 3, 6, 2), (600, 2, 9, 3), (7, 5, 5, 3)]
 
 
