@@ -231,6 +231,7 @@ __global__ void __launch_bounds__(32 * TOUR_WARPS) tour_edges_kernel(TourEdgeArg
             const unsigned si = S[i], sn = i + 1 < L ? S[i + 1] : TOUR_INF;
             const int e = si < sn ? (int)si : (si >= (unsigned)L ? L - 1 : (int)si - 1);
             const int len = e - i + 1;
+            if (len > plen) continue;  // a longer one comes before p
             const unsigned long long raw = Pf[e + 1] - Pf[i] * a.pw[len];
             const unsigned long long h = hash_key(raw, gi, len);
             long long j = (long long)(h & (unsigned long long)tmask);
@@ -240,10 +241,11 @@ __global__ void __launch_bounds__(32 * TOUR_WARPS) tour_edges_kernel(TourEdgeArg
                 if (kj != h) continue;
                 const long long q = tidx[j];
                 if (q < lo || q >= hi) continue;
+                // q comes after p: shorter, or as long and later in canonical order
+                if (len == plen && q <= p) continue;
                 const long long qo = a.pp_off[q];
                 if (a.pp_off[q + 1] - qo != len || !same_seq(a.pp_vert + qo, t + i, len)) continue;
-                // q comes after p: shorter, or as long and later in canonical order
-                if (len < plen || (len == plen && q > p)) hit[atomicAdd(&s_nhit[wid], 1)] = (int)q;
+                hit[atomicAdd(&s_nhit[wid], 1)] = (int)q;
                 break;
             }
         }
