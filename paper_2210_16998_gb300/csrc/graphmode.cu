@@ -19,6 +19,7 @@ namespace {
 constexpr int GMB = 256;      // threads per block of the streaming kernels
 constexpr int GM_SCAN_ITEMS = 8;
 constexpr long long GM_SCAN_TILE = (long long)GMB * GM_SCAN_ITEMS;
+constexpr long long GM_SCAN_FEW_TILES = 4096;  // above, the tile sums get a scan of their own
 
 __device__ __forceinline__ long long clampc(long long v, long long cap) { return v < 0 ? 0 : (v > cap ? cap : v); }
 
@@ -42,8 +43,7 @@ __global__ void __launch_bounds__(GMB) gm_scan_reduce(const T *in, const long lo
     }
 }
 
-__global__ void __launch_bounds__(GMB) gm_scan_tiles(long long *tile_sums, const long long *n_dev, long long n_cap,
-                                                     long long *total_out) {
+__global__ void __launch_bounds__(GMB) gm_scan_tiles(long long *tile_sums, const long long *n_dev, long long n_cap) {
     const long long n = clampc(*n_dev, n_cap);
     const long long ntiles = (n + GM_SCAN_TILE - 1) / GM_SCAN_TILE;
     long long carry = 0;
@@ -55,19 +55,26 @@ __global__ void __launch_bounds__(GMB) gm_scan_tiles(long long *tile_sums, const
         if (i < ntiles) tile_sums[i] = carry + ex;
         carry += total;
     }
-    if (threadIdx.x == 0) {
-        tile_sums[ntiles] = carry;
-        if (total_out) *total_out = carry;
-    }
+    if (threadIdx.x == 0) tile_sums[ntiles] = carry;
 }
 
-template <typename T>
+// RAW: tile_sums holds the sums themselves (few tiles: each adds up those
+// before it), else their prefix
+template <typename T, bool RAW>
 __global__ void __launch_bounds__(GMB) gm_scan_down(const T *in, long long *out, const long long *n_dev,
                                                     long long n_cap, const long long *tile_sums) {
     const long long n = clampc(*n_dev, n_cap);
     const long long ntiles = (n + GM_SCAN_TILE - 1) / GM_SCAN_TILE;
+    if (RAW && ntiles == 0 && blockIdx.x == 0 && threadIdx.x == 0) out[0] = 0;
     for (long long t = blockIdx.x; t < ntiles; t += gridDim.x) {
         const long long base = t * GM_SCAN_TILE + (long long)threadIdx.x * GM_SCAN_ITEMS;
+        long long before = 0;
+        if constexpr (RAW) {
+            for (long long i = threadIdx.x; i < t; i += GMB) before += tile_sums[i];
+            block_excl_scan_i64<GMB>(before, before);
+        } else {
+            before = tile_sums[t];
+        }
         long long v[GM_SCAN_ITEMS];
         long long s = 0;
 #pragma unroll
@@ -77,15 +84,16 @@ __global__ void __launch_bounds__(GMB) gm_scan_down(const T *in, long long *out,
             s += v[j];
         }
         long long total;
-        long long run = block_excl_scan_i64<GMB>(s, total) + tile_sums[t];
+        long long run = block_excl_scan_i64<GMB>(s, total) + before;
 #pragma unroll
         for (int j = 0; j < GM_SCAN_ITEMS; ++j) {
             const long long i = base + j;
             if (i < n) out[i] = run;
             run += v[j];
         }
+        if (RAW && t == ntiles - 1 && threadIdx.x == 0) out[n] = before + total;
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) out[n] = tile_sums[ntiles];
+    if (!RAW && blockIdx.x == 0 && threadIdx.x == 0) out[n] = tile_sums[ntiles];
 }
 
 // ---------------------------------------------------------------------------
@@ -263,11 +271,16 @@ unsigned stream_grid(int num_sms) { return (unsigned)(num_sms * 8); }
 
 template <typename T>
 cudaError_t gm_scan(const T *in, long long *out, const long long *n_dev, long long n_cap, long long *tmp,
-                    long long *total_out, int num_sms, cudaStream_t s) {
+                    int num_sms, cudaStream_t s) {
     const unsigned grid = stream_grid(num_sms);
     gm_scan_reduce<T><<<grid, GMB, 0, s>>>(in, n_dev, n_cap, tmp);
-    gm_scan_tiles<<<1, GMB, 0, s>>>(tmp, n_dev, n_cap, total_out);
-    gm_scan_down<T><<<grid, GMB, 0, s>>>(in, out, n_dev, n_cap, tmp);
+    if (n_cap <= GM_SCAN_FEW_TILES * GM_SCAN_TILE) {
+        gm_scan_down<T, true><<<grid, GMB, 0, s>>>(in, out, n_dev, n_cap, tmp);
+        note_launch(2);
+        return cudaGetLastError();
+    }
+    gm_scan_tiles<<<1, GMB, 0, s>>>(tmp, n_dev, n_cap);
+    gm_scan_down<T, false><<<grid, GMB, 0, s>>>(in, out, n_dev, n_cap, tmp);
     note_launch(3);
     return cudaGetLastError();
 }
@@ -309,14 +322,14 @@ cudaError_t gm_enqueue_tp(const GmArgs &a, cudaStream_t s) {
     gm_tp_len<<<grid, GMB, 0, s>>>(a);
     note_launch();
     cudaError_t e;
-    if ((e = gm_scan<long long>(a.tp_len, a.tp_off0, &a.counts->P, a.P_cap, a.scan_tmp, nullptr, a.num_sms, s)))
+    if ((e = gm_scan<long long>(a.tp_len, a.tp_off0, &a.counts->P, a.P_cap, a.scan_tmp, a.num_sms, s)))
         return e;
-    if ((e = gm_scan<long long>(a.len, a.key_off, &a.counts->P, a.P_cap, a.scan_tmp, nullptr, a.num_sms, s)))
+    if ((e = gm_scan<long long>(a.len, a.key_off, &a.counts->P, a.P_cap, a.scan_tmp, a.num_sms, s)))
         return e;
     gm_tp_check<<<1, 32, 0, s>>>(a);
     gm_order_mark<<<grid, GMB, 0, s>>>(a);
     note_launch(2);
-    if ((e = gm_scan<int>(a.order.start, a.order.sub_rank, &a.counts->P, a.P_cap, a.scan_tmp, nullptr, a.num_sms, s)))
+    if ((e = gm_scan<int>(a.order.start, a.order.sub_rank, &a.counts->P, a.P_cap, a.scan_tmp, a.num_sms, s)))
         return e;
     if ((e = cudaMemsetAsync(a.order.slot_n, 0, sizeof(long long) * (a.slots + 1), s))) return e;
     gm_order_list<<<grid, GMB, 0, s>>>(a);
@@ -335,9 +348,9 @@ cudaError_t gm_enqueue_tp(const GmArgs &a, cudaStream_t s) {
     if (a.key_bits == 8) gm_tp_dedup<8><<<grid, GMB, 0, s>>>(a);
     else gm_tp_dedup<16><<<grid, GMB, 0, s>>>(a);
     note_launch(a.tp_rounds + 1);
-    if ((e = gm_scan<long long>(a.tp_len, a.keep_off, &a.counts->P, a.P_cap, a.scan_tmp, nullptr, a.num_sms, s)))
+    if ((e = gm_scan<long long>(a.tp_len, a.keep_off, &a.counts->P, a.P_cap, a.scan_tmp, a.num_sms, s)))
         return e;
-    if ((e = gm_scan<int>(a.keep, a.keep_rank, &a.counts->P, a.P_cap, a.scan_tmp, nullptr, a.num_sms, s)))
+    if ((e = gm_scan<int>(a.keep, a.keep_rank, &a.counts->P, a.P_cap, a.scan_tmp, a.num_sms, s)))
         return e;
     gm_tp_totals<<<1, 32, 0, s>>>(a);
     if (a.key_bits == 8) gm_tp_gather<unsigned char><<<grid, GMB, 0, s>>>(a);
