@@ -428,6 +428,7 @@ struct tpg_cfg {
     long long last_edges = 0;  // cover edges of the last touring call
     cudaEvent_t ev[12] = {};  // [8], [9]: host-result copies; [10], [11]: touring
     long long last_tv0 = 0;  // TP vertices before dedup in the last tpg_test_paths
+    int max_tp = 0;          // vertices of the longest TP of the last call
 
     // graph mode: the whole hot path captured in one CUDA graph
     struct GraphPlan {
@@ -1392,7 +1393,7 @@ int run_test_paths_small(tpg_cfg *g, Block **o_off, Block **o_vert, Block **o_gp
         a.result = g->ctl.as<long long>();
         cudaEventRecord(g->ev[4], s);
         if (cuda_err(tp_small(a, s)) ||
-            cuda_err(cudaMemcpyAsync(h, a.result, 4 * sizeof(long long), cudaMemcpyDeviceToHost, s)))
+            cuda_err(cudaMemcpyAsync(h, a.result, 5 * sizeof(long long), cudaMemcpyDeviceToHost, s)))
             rc = TPG_ECUDA;
         cudaEventRecord(g->ev[5], s);
         if (cudaStreamSynchronize(s) != cudaSuccess && rc == TPG_OK) rc = TPG_ECUDA;
@@ -1400,6 +1401,7 @@ int run_test_paths_small(tpg_cfg *g, Block **o_off, Block **o_vert, Block **o_gp
     if (rc == TPG_OK && (h[0] & ERR_UNREACH)) rc = TPG_EUNREACH;
     if (rc == TPG_OK) {
         g->last_tv0 = h[1];
+        g->max_tp = (int)h[4];
         *oT = h[2];
         *oTV = h[3];
         if (h[1] == g->V) {  // every TP is its PP: the PP list's blocks serve both
@@ -1465,7 +1467,7 @@ int run_test_paths(tpg_cfg *g, Block **o_off, Block **o_vert, Block **o_gptr, lo
     RC(ensure(g, g->s_tmp, sizeof(long long) * scan_tmp_elems(std::max<long long>(P, g->M + g->N) + 1)));
     RC(ensure(g, g->ctl, CTL_BYTES));
     CK(cudaEventRecord(g->ev[4], s));
-    CK(cudaMemsetAsync(g->ctl.p, 0, 4 * sizeof(long long), s));  // error word, -, runs, graphs with PPs
+    CK(cudaMemsetAsync(g->ctl.p, 0, 5 * sizeof(long long), s));  // error word, -, runs, graphs with PPs, longest TP
     long long *tp_len = g->s_i64[0].as<long long>();
     CK(tp_lengths(pp_off, g->pp_ends.as<int2>(), pp_graph, P, g->gd, tp_len, g->ctl.as<int>(),
                   g->ctl.as<unsigned long long>() + 2, s));
@@ -1481,12 +1483,13 @@ int run_test_paths(tpg_cfg *g, Block **o_off, Block **o_vert, Block **o_gptr, lo
         long long *tmp = g->s_tmp.as<long long>();
         if (cuda_err(scan_i64_sums(tp_len, P, tmp, s))) { rc = TPG_ECUDA; break; }
         cudaMemcpyAsync(h, tmp + scan_total_index(P), sizeof(long long), cudaMemcpyDeviceToHost, s);
-        cudaMemcpyAsync(h + 1, g->ctl.p, 4 * sizeof(long long), cudaMemcpyDeviceToHost, s);
+        cudaMemcpyAsync(h + 1, g->ctl.p, 5 * sizeof(long long), cudaMemcpyDeviceToHost, s);
         if (cudaStreamSynchronize(s) != cudaSuccess) { rc = TPG_ECUDA; break; }
         TV = h[0];
         g->last_tv0 = TV;
         if (((int *)(h + 1))[0] & ERR_UNREACH) { rc = TPG_EUNREACH; break; }
         const long long runs = h[3], graphs_with_pp = h[4];
+        g->max_tp = (int)h[5];
         if (TV != g->V && cuda_err(scan_i64_finish(tp_len, (long long *)tp_off->p, P, tmp, s))) {
             rc = TPG_ECUDA;
             break;
@@ -2149,6 +2152,7 @@ static int run_touring(tpg_cfg *g, Block *toff, Block *tvert, Block *tgptr, long
             a.edge_count = ecount;
             a.err = err;
             a.maxn = g->maxn;
+            a.max_tp = std::max(g->max_tp, 1);  // (of the call that made toff)
             if ((rc = cuda_err(tour_edges(a, g->num_sms, &warps, s)))) break;
             if ((rc = cuda_err(cudaMemcpyAsync(h, ecount, sizeof(long long), cudaMemcpyDeviceToHost, s))) ||
                 (rc = cuda_err(cudaMemcpyAsync(h + 1, err, sizeof(int), cudaMemcpyDeviceToHost, s))) ||

@@ -24,12 +24,13 @@ static unsigned grid_for(long long n, int block = 256) {
 
 // TP lengths from each PP's (first, last) local vertex, which the
 // materialisation wrote beside the PP list (coalesced reads only); runs[0] +=
-// runs of PPs with one first vertex, runs[1] += graphs that own a PP.
+// runs of PPs with one first vertex, runs[1] += graphs that own a PP, runs[2] =
+// the longest.
 __global__ void __launch_bounds__(256) tp_len_kernel(const long long *__restrict__ pp_off,
                                                      const int2 *__restrict__ pp_ends,
                                                      const int *__restrict__ pp_graph, long long P, GraphDev g,
                                                      long long *tp_len, int *err, unsigned long long *runs) {
-    int nruns = 0, ngraphs = 0;
+    int nruns = 0, ngraphs = 0, longest = 0;
     for (long long i = blockIdx.x * 256ll + threadIdx.x; i < P; i += gridDim.x * 256ll) {
         const long long o0 = pp_off[i], o1 = pp_off[i + 1];
         const int gid = pp_graph ? pp_graph[i] : 0;
@@ -41,15 +42,19 @@ __global__ void __launch_bounds__(256) tp_len_kernel(const long long *__restrict
         if (pl == 0 || sl == 0) atomicOr(err, ERR_UNREACH);
         else len = (long long)(pl - 1) + (o1 - o0) + (sl - 1);
         tp_len[i] = len;
+        longest = len > longest ? (int)len : longest;
         const bool new_graph = i == 0 || (pp_graph && pp_graph[i - 1] != gid);
         ngraphs += new_graph;
         nruns += new_graph || pp_ends[i - 1].x != e.x;
     }
     nruns = __reduce_add_sync(0xffffffffu, nruns);
     ngraphs = __reduce_add_sync(0xffffffffu, ngraphs);
-    if ((threadIdx.x & 31) == 0 && nruns) {
-        atomicAdd(runs, (unsigned long long)nruns);
+    longest = __reduce_max_sync(0xffffffffu, longest);
+    if ((threadIdx.x & 31) == 0 && longest) {
+        if (nruns) atomicAdd(runs, (unsigned long long)nruns);
         if (ngraphs) atomicAdd(runs + 1, (unsigned long long)ngraphs);
+        if ((unsigned long long)longest > *(volatile unsigned long long *)(runs + 2))
+            atomicMax(runs + 2, (unsigned long long)longest);
     }
 }
 
@@ -399,11 +404,11 @@ __device__ __forceinline__ long long tps_scan(long long n, long long *out, F f) 
 template <typename T>
 __global__ void __launch_bounds__(TPS_BLOCK) tp_small_kernel(TpSmallArgs a) {
     constexpr int BITS = 8 * sizeof(T);
-    __shared__ int s_err;
+    __shared__ int s_err, s_longest;
     const TpOrder &o = a.o;
     const GraphDev &g = o.g;
     const long long P = a.P, tid = threadIdx.x;
-    if (tid == 0) s_err = 0;
+    if (tid == 0) s_err = s_longest = 0;
     __syncthreads();
     const long long TV = tps_scan(P, a.tp_off, [&](long long i) {
         const int2 e = a.ends[i];
@@ -411,8 +416,10 @@ __global__ void __launch_bounds__(TPS_BLOCK) tp_small_kernel(TpSmallArgs a) {
         if (pl == 0 || sl == 0) s_err = ERR_UNREACH;
         const long long len = pl == 0 || sl == 0 ? 0 : (long long)(pl - 1) + (o.pp_off[i + 1] - o.pp_off[i]) + (sl - 1);
         a.tp_len[i] = len;
+        atomicMax(&s_longest, (int)len);
         return len;
     });
+    if (tid == 0) a.result[4] = s_longest;
     if (s_err || TV == a.V) {  // (equal: every TP is its PP)
         if (tid == 0) {
             a.result[0] = s_err;

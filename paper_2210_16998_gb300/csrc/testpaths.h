@@ -48,8 +48,8 @@ cudaError_t tp_index_map(const long long *perm, const int *keep, const long long
                          cudaStream_t s);
 
 // The whole of it for P TPs (P > 0) of one graph, in one block: result = {error
-// word, TP vertices before dedup, TPs, their vertices}, the last two and all
-// lists only if the first is 0 and the second is not V (the PPs' vertices).
+// word, TP vertices before dedup, TPs, their vertices, the longest TP}, the third,
+// the fourth and all lists only if the first is 0 and the second is not V (the PPs' vertices).
 // o as for the steps above, with room for P sub-runs; final_off[P + 1],
 // out_vert for the vertices before dedup, pp_to_tp (tp_index_map) may be null.
 struct TpSmallArgs {

@@ -39,7 +39,7 @@ struct TourEdgeArgs {
     long long edge_cap;
     unsigned long long *edge_count;  // zero at launch; counts every edge, also past edge_cap
     int *err;                  // ERR_* flags
-    int maxn;
+    int maxn, max_tp;  // vertices of the largest graph, of the longest TP
 };
 // one launch, every PP of every graph (persistent warps, as many as fit
 // num_sms SMs); *warps_out receives the warps per block
