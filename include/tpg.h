@@ -85,12 +85,12 @@ typedef struct tpg_paths {
 
 /* Statistics of the last tpg_prime_paths call on a handle. */
 typedef struct tpg_stats {
-    int64_t simple_paths;       /* frontier nodes enumerated (simple paths incl. closed cycles) */
+    int64_t simple_paths;       /* simple paths incl. closed cycles (those that cannot begin a PP are counted, not stored) */
     int64_t prime_paths;        /* P */
     int64_t pp_vertices;        /* total vertex ids in the PP list */
-    int32_t levels;             /* frontier levels processed */
+    int32_t levels;             /* vertices of the longest simple path */
     int32_t pp_levels;          /* levels that held at least one PP */
-    int64_t peak_level_nodes;   /* largest frontier level */
+    int64_t peak_level_nodes;   /* most simple paths of one length */
     int64_t arena_bytes_used;   /* persistent path arena bytes written */
     int64_t arena_bytes_alloc;  /* path arena bytes allocated */
     int64_t frontier_bytes_alloc; /* ping-pong frontier bytes allocated */

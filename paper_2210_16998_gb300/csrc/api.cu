@@ -415,7 +415,7 @@ struct tpg_cfg {
     int split = 1;  // work units per chunk of the frontier kernel
     unsigned long long spin_ns = SPIN_LIMIT_NS;  // limit of each grid-barrier wait of the frontier launch
     // generic scratch
-    DevBuf s_keys[2], s_refs[2], s_len, s_tmp, s_i32[3], s_i64[4];
+    DevBuf s_refs[2], s_len, s_tmp, s_i32[3], s_i64[3];
     DevBuf pp_ends;  // (first, last) local vertex of each cached PP, for the TP lengths
     DevBuf tp_key_off, tp_key;  // packed comparison keys of the TPs being sorted
 
@@ -436,7 +436,7 @@ struct tpg_cfg {
         cudaGraphExec_t exec = nullptr;
         cudaStream_t own_stream = nullptr;
         DevBuf seg, ppseg, tfl[2], tvis[2], tcnt[2];
-        DevBuf lvl_pp_off, refs[2], len, scan_tmp, pp_graph, tp_len, tp_start, sub_rank, pos_sub, subs, slots,
+        DevBuf refs, len, scan_tmp, pp_graph, tp_len, tp_start, sub_rank, pos_sub, subs, slots,
             tp_off0, perm[2], keep, keep_off, keep_rank, tp_graph, counts,
             key_off, key;
         Block *pp_off = nullptr, *pp_vert = nullptr, *pp_gptr = nullptr;
@@ -514,8 +514,8 @@ void release_plan(tpg_cfg *g) {
     auto &p = g->gp;
     if (p.exec) cudaGraphExecDestroy(p.exec);
     p.exec = nullptr;
-    DevBuf *all[] = {&p.seg, &p.ppseg, &p.tfl[0], &p.tfl[1], &p.tvis[0], &p.tvis[1], &p.tcnt[0], &p.tcnt[1], &p.lvl_pp_off,
-                     &p.refs[0], &p.refs[1], &p.len, &p.scan_tmp, &p.pp_graph, &p.tp_len,
+    DevBuf *all[] = {&p.seg, &p.ppseg, &p.tfl[0], &p.tfl[1], &p.tvis[0], &p.tvis[1], &p.tcnt[0], &p.tcnt[1],
+                     &p.refs, &p.len, &p.scan_tmp, &p.pp_graph, &p.tp_len,
                      &p.tp_start, &p.sub_rank, &p.pos_sub, &p.subs, &p.slots, &p.tp_off0,
                      &p.perm[0], &p.perm[1], &p.keep, &p.keep_off, &p.keep_rank, &p.tp_graph,
                      &p.counts, &p.key_off, &p.key};
@@ -538,9 +538,9 @@ void destroy_cfg(tpg_cfg *g) {
                      &g->tbl_base, &g->dist, &g->pred, &g->pre_len, &g->suf_len, &g->pre_off, &g->suf_off,
                      &g->smask, &g->pmask, &g->arc_slot, &g->end_slot, &g->thin, &g->tp_subs, &g->tp_slots, &g->cmask, &g->dflags, &g->xinfo, &g->dropD, &g->dropX, &g->drop_lvl,
                      &g->pre_seq, &g->suf_seq, &g->tfl[0], &g->tfl[1], &g->tvis[0], &g->tvis[1], &g->tcnt[0], &g->tcnt[1],
-                     &g->levels, &g->agg, &g->ctl, &g->s_keys[0], &g->s_keys[1],
+                     &g->levels, &g->agg, &g->ctl, 
                      &g->s_refs[0], &g->s_refs[1], &g->s_len, &g->s_tmp, &g->s_i32[0], &g->s_i32[1],
-                     &g->s_i32[2], &g->s_i64[0], &g->s_i64[1], &g->s_i64[2], &g->s_i64[3], &g->pp_ends, &g->tp_key_off, &g->tp_key,
+                     &g->s_i32[2], &g->s_i64[0], &g->s_i64[1], &g->s_i64[2], &g->pp_ends, &g->tp_key_off, &g->tp_key,
                      &g->trace};
     for (DevBuf *b : all) release(g, *b);
     for (auto &b : g->node_segs) release(g, b);
@@ -1672,10 +1672,9 @@ int capture_plan(tpg_cfg *g) {
         RC(ensure(g, p.tfl[b], sizeof(int2) * p.lvl_cap));
         RC(ensure(g, p.tvis[b], sizeof(unsigned) * (size_t)W * p.lvl_cap));
         RC(ensure(g, p.tcnt[b], sizeof(unsigned short) * p.lvl_cap));
-        RC(ensure(g, p.refs[b], sizeof(long long) * Pc));
         RC(ensure(g, p.perm[b], sizeof(long long) * Pc));
     }
-    RC(ensure(g, p.lvl_pp_off, sizeof(long long) * (g->max_levels + 1)));
+    RC(ensure(g, p.refs, sizeof(long long) * Pc));
     RC(ensure(g, p.len, sizeof(long long) * Pc));
     RC(ensure(g, p.scan_tmp, sizeof(long long) * std::max(gm_scan_tmp_elems(Pc + 1), scan_tmp_elems(g->M + g->N + 1))));
     RC(ensure(g, p.pp_graph, sizeof(int) * Pc));
@@ -1744,8 +1743,7 @@ int capture_plan(tpg_cfg *g) {
     m.TV_cap = p.TV_cap;
     m.num_sms = g->num_sms;
     m.tp_rounds = gm_tp_rounds(g->maxn);
-    m.lvl_pp_off = p.lvl_pp_off.as<long long>();
-    for (int b = 0; b < 2; ++b) m.refs[b] = p.refs[b].as<long long>();
+    m.refs = p.refs.as<long long>();
     m.len = p.len.as<long long>();
     m.scan_tmp = p.scan_tmp.as<long long>();
     m.pp_off = (long long *)p.pp_off->p;

@@ -108,14 +108,12 @@ __global__ void __launch_bounds__(GMB) gm_level_summary(GmArgs a) {
         long long v = 0;
         if (ok && k >= 1 && k < ml) v = a.levels[k].count > 0 ? a.levels[k].pp_count : 0;
         long long total, vtotal;
-        const long long ex = block_excl_scan_i64<GMB>(v, total);
+        block_excl_scan_i64<GMB>(v, total);
         block_excl_scan_i64<GMB>(v * k, vtotal);
-        if (k < ml) a.lvl_pp_off[k] = carry + ex;
         carry += total;
         vcarry += vtotal;
     }
     if (threadIdx.x == 0) {
-        a.lvl_pp_off[ml] = carry;
         GmCounts *c = a.counts;
         c->P = carry;
         c->V = vcarry;
@@ -140,7 +138,7 @@ __global__ void __launch_bounds__(GM_MAT_WARPS * 32, 8) gm_materialize(GmArgs a)
     __shared__ int2 *s_nodes[MAT_MAX_LV];
     int2 *const *lv = cache_level_nodes(a.levels, a.max_levels, s_nodes);
     const long long P = gm_P(a);
-    materialize_warps<GM_MAT_WARPS, CH, T>(a.refs[a.counts->pp_buf], nullptr, 0, P, a.pp_off, a.levels, a.g,
+    materialize_warps<GM_MAT_WARPS, CH, T>(a.refs, nullptr, 0, P, a.pp_off, a.levels, a.g,
                                            a.pp_vert, a.g.G > 1 ? a.pp_graph : nullptr, sbuf, lv);
 }
 
@@ -302,7 +300,7 @@ cudaError_t gm_enqueue_pp(const GmArgs &a, cudaStream_t s) {
     PlaceArgs r{};
     r.levels = a.levels;
     r.max_levels = a.max_levels;
-    r.refs = a.refs[0];  // counts->pp_buf stays 0
+    r.refs = a.refs;
     r.off = a.pp_off;
     r.cap = a.P_cap;
     r.skip = &a.counts->flags;

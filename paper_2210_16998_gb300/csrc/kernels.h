@@ -198,7 +198,6 @@ static_assert(GM_TIMEOUT == 16, "flag bits must stay distinct");
 struct GmCounts {
     long long P, V, TV0, T, TV;
     int flags;
-    int pp_buf;  // which keys/refs buffer holds the ordered PPs
 };
 struct GmArgs {
     GraphDev g;
@@ -207,8 +206,7 @@ struct GmArgs {
     const int *enum_err;
     long long P_cap, V_cap, TV0_cap, TV_cap;
     int num_sms, tp_rounds;
-    long long *lvl_pp_off;  // [max_levels+1]
-    long long *refs[2];
+    long long *refs;        // [P_cap] the ordered PPs: level << 32 | node
     long long *len;         // [P_cap]
     long long *scan_tmp;    // gm_scan_tmp_elems(P_cap)
     long long *pp_off;      // [P_cap+1]
