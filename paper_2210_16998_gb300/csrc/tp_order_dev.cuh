@@ -110,23 +110,28 @@ __device__ __forceinline__ int tp_slot_of(const TpOrder &o, long long i, int *le
     const int gid = o.pp_graph ? o.pp_graph[i] : 0;
     const int vb = g.vgraph ? g.vbase[gid] : 0, n = (g.vgraph ? g.vbase[gid + 1] : g.N) - vb;
     const int *prow = g.pred + g.tbl_base[gid] + (long long)(g.entry[gid] - vb) * n;
+    // along seq[p .. end) as long as its arcs are the tree's, four at a time (a
+    // step is two dependent loads); y: the vertex that another arc leads to
     int x = o.pp_vert[o0], y = -1;
-    for (long long p = o0 + 1; p < o1; ++p) {
-        y = o.pp_vert[p];
-        if (prow[y] != x) break;
-        x = y;
-        y = -1;
-    }
+    auto follow = [&](const int *seq, long long p, long long end) {
+        for (; p < end && y < 0; p += 4) {
+            int v[4], pr[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) v[j] = p + j < end ? seq[p + j] : -1;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) pr[j] = v[j] >= 0 ? prow[v[j]] : -1;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                if (y >= 0 || v[j] < 0) continue;
+                if (pr[j] == x) x = v[j];
+                else y = v[j];
+            }
+        }
+    };
+    follow(o.pp_vert, o0 + 1, o1);
     if (y < 0) {  // the PP ends on the tree: on along path(last vertex -> exit)
         const int last = x + vb;
-        const int *suf = g.suf_seq + g.suf_off[last];
-        const int sl = g.suf_len[last];
-        for (int p = 1; p < sl; ++p) {
-            y = suf[p];
-            if (prow[y] != x) break;
-            x = y;
-            y = -1;
-        }
+        follow(g.suf_seq + g.suf_off[last], 1, g.suf_len[last]);
     }
     *len = g.pre_len[x + vb] + (y >= 0 ? 1 : 0);
     const int base = g.rp[vb] + vb;
